@@ -6,10 +6,10 @@
 //  forward  persistent CTAs of 128 threads over rounds of 32 samples, layer
 //           by layer on the tcgen05 tensor cores (initnet_tc.cuh: BF16
 //           operands in shared memory, FP32 accumulators in tensor memory)
-//  train    the forward pass of one sample per warp (same layers, BF16
-//           activations), then the backward pass in FP32 per warp, with
-//           the weight gradients summed in shared memory per CTA and added to
-//           the global gradient once per CTA
+//  train    two samples per CTA at a time through the forward pass (same
+//           layers, BF16 activations) and the backward pass in FP32, with
+//           the weight gradients summed in registers over the CTA's samples
+//           and added to the global gradient once per CTA
 //  adam     Adam update of the master parameters
 #include <math.h>
 
@@ -267,14 +267,13 @@ extern "C" vio_status vio_initnet_train_step(const void* d_packed, const uint16_
     return VIO_ERR_INVALID_ARG;
   if (n == 0) return VIO_OK;
   const int smem = vio::initnet_train_smem();
-  cudaError_t e = cudaFuncSetAttribute(vio::train_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return VIO_ERR_CUDA;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int blocks = (int)std::min<long long>((long long)sms, (n + vio::TRAIN_WARPS - 1) /
-                                                                  vio::TRAIN_WARPS);
+  static vio::PerDeviceOnce attr;
+  if (vio::once_per_device(attr, [&] {
+        return cudaFuncSetAttribute(vio::train_kernel,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      }) != cudaSuccess)
+    return VIO_ERR_CUDA;
+  const int blocks = vio::train_blocks(n, vio::sm_count());
   vio::train_kernel<<<blocks, vio::TRAIN_WARPS * 32, smem, (cudaStream_t)stream>>>(
       d_packed, d_x, d_flow, d_index, n, grad_scale, label_radius, d_grad, d_loss);
   return cudaGetLastError() == cudaSuccess ? VIO_OK : VIO_ERR_CUDA;

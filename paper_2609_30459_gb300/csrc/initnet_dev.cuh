@@ -7,13 +7,13 @@
 // fully connected 128 -> 64 with ReLU, then 64 -> 3: flow = 16 px * (o0, o1)
 // and confidence = sigmoid(o2).
 //
-// One warp evaluates one sample on the tensor cores: every layer is a GEMM
-// (output positions x input taps) x (input taps x output channels) done with
-// mma.sync m16n8k16 on BF16 operands and FP32 accumulators. Activations live
-// in the warp's shared memory as BF16 with a zero border, so the im2col
-// offset of (position, tap) splits into a per-row base plus a per-column
-// offset and needs no bounds test. Weights are packed as BF16 [N][K] rows
-// (K padded to a multiple of 16) so a B fragment is one 32-bit load.
+// The training pass runs every layer as a GEMM (output positions x input taps)
+// x (input taps x output channels) with mma.sync m16n8k16 on BF16 operands and
+// FP32 accumulators. Activations live in shared memory as BF16 with a zero
+// border, so the im2col offset of (position, tap) splits into a per-row base
+// plus a per-column offset and needs no bounds test. Weights are packed as BF16
+// [N][K] rows (K padded to a multiple of 16) so a B fragment is one 32-bit
+// load.
 #pragma once
 #include <cuda_bf16.h>
 
@@ -88,78 +88,6 @@ __device__ __forceinline__ int tap_off(int k, int ntaps, int P) {
   return c * P * P + u * P + v;
 }
 
-// 3x3 stride-2 convolution + bias + ReLU of a bordered BF16 map
-// [CIN][HIN+2][HIN+2] into a bordered map [32][HOUT+2][HOUT+2] (or, when
-// flat_out, into a plain [32*HOUT*HOUT] vector in (channel, row, col) order).
-template <int CIN, int HIN, int KPAD, bool FLAT_OUT>
-__device__ __forceinline__ void conv_layer(const uint16_t* in, uint16_t* out, const uint16_t* zero,
-                                           const uint16_t* W, const float* bias, int lane) {
-  constexpr int HOUT = HIN / 2;
-  constexpr int P = HIN + 2, PO = HOUT + 2;
-  constexpr int M = HOUT * HOUT;
-  constexpr int MT = (M + 15) / 16;
-  constexpr int NTAPS = CIN * 9;
-  const int g = lane >> 2, t = lane & 3;
-#pragma unroll 1
-  for (int mt = 0; mt < MT; ++mt) {
-    // the two output positions (rows) of this thread in the tile
-    int base[2];
-    bool live[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = mt * 16 + g + 8 * h;
-      live[h] = r < M;
-      const int i = live[h] ? r / HOUT : 0, j = live[h] ? r % HOUT : 0;
-      base[h] = 2 * i * P + 2 * j;     // bordered coordinates of tap (0, 0)
-    }
-    float acc[4][4];
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-#pragma unroll 2
-    for (int ks = 0; ks < KPAD / 16; ++ks) {
-      int off[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) off[q] = tap_off(ks * 16 + 2 * t + (q & 1) + 8 * (q >> 1),
-                                                   NTAPS, P);
-      uint32_t a[4];
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const int q0 = 2 * half, q1 = 2 * half + 1;
-          const uint16_t lo = (live[h] && off[q0] >= 0) ? in[base[h] + off[q0]] : zero[0];
-          const uint16_t hi = (live[h] && off[q1] >= 0) ? in[base[h] + off[q1]] : zero[0];
-          a[h + 2 * half] = (uint32_t)lo | ((uint32_t)hi << 16);
-        }
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        const uint16_t* wr = W + (nt * 8 + g) * KPAD + ks * 16 + 2 * t;
-        const uint32_t b0 = __ldg(reinterpret_cast<const uint32_t*>(wr));
-        const uint32_t b1 = __ldg(reinterpret_cast<const uint32_t*>(wr + 8));
-        mma16816(acc[nt], a, b0, b1);
-      }
-    }
-    // epilogue: bias, ReLU, BF16
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int r = mt * 16 + g + 8 * (e >> 1);
-        const int n = nt * 8 + 2 * t + (e & 1);
-        if (r < M) {
-          const float v = fmaxf(acc[nt][e] + bias[n], 0.f);
-          const int i = r / HOUT, j = r % HOUT;
-          if (FLAT_OUT)
-            out[n * M + r] = f2bf(v);
-          else
-            out[n * PO * PO + (i + 1) * PO + (j + 1)] = f2bf(v);
-        }
-      }
-  }
-}
-
 // Fully connected layer on one input vector (row 0 of a 16-row tile):
 // out[n] = act(sum_k W[n][k] in[k] + b[n]) for n < NOUT; returns outputs in
 // FP32 through `res` (thread-local: lanes with g == 0 hold row 0).
@@ -194,46 +122,6 @@ __device__ __forceinline__ void clear_warp_smem(uint8_t* ws, int lane) {
   uint32_t* p = reinterpret_cast<uint32_t*>(ws);
   for (int i = lane; i < WARP_SMEM / 4; i += 32) p[i] = 0u;
   __syncwarp();
-}
-
-// Forward pass of one sample whose input is in ws + S_X (bordered, BF16).
-// Returns o[0..2] (raw outputs) in every lane.
-__device__ __forceinline__ void forward_warp(const Packed& P, uint8_t* ws, int lane, float* o) {
-  uint16_t* x = reinterpret_cast<uint16_t*>(ws + S_X);
-  uint16_t* h1 = reinterpret_cast<uint16_t*>(ws + S_H1);
-  uint16_t* h2 = reinterpret_cast<uint16_t*>(ws + S_H2);
-  uint16_t* h3 = reinterpret_cast<uint16_t*>(ws + S_H3);
-  uint16_t* h4 = reinterpret_cast<uint16_t*>(ws + S_H4);
-  const uint16_t* zero = reinterpret_cast<const uint16_t*>(ws + S_ZERO);
-  conv_layer<4, 16, K1, false>(x, h1, zero, P.w + OFF_W1, P.b + OFF_B1, lane);
-  __syncwarp();
-  conv_layer<32, 8, K2, false>(h1, h2, zero, P.w + OFF_W2, P.b + OFF_B2, lane);
-  __syncwarp();
-  conv_layer<32, 4, K3, true>(h2, h3, zero, P.w + OFF_W3, P.b + OFF_B3, lane);
-  __syncwarp();
-  const int g = lane >> 2, t = lane & 3;
-  {
-    float acc[8][4];
-    fc_layer<K4, 8>(h3, P.w + OFF_W4, lane, acc);
-    if (g == 0)
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int n = nt * 8 + 2 * t + e;
-          h4[n] = f2bf(fmaxf(acc[nt][e] + P.b[OFF_B4 + n], 0.f));
-        }
-  }
-  __syncwarp();
-  float acc5[1][4];
-  fc_layer<K5, 1>(h4, P.w + OFF_W5, lane, acc5);
-  // row 0, columns 2t, 2t+1 live in lane t (g == 0): outputs 0..2 in lanes 0, 1
-  const float v0 = acc5[0][0], v1 = acc5[0][1];
-  const float a0 = __shfl_sync(0xffffffffu, v0, 0), a1 = __shfl_sync(0xffffffffu, v1, 0);
-  const float a2 = __shfl_sync(0xffffffffu, v0, 1);
-  o[0] = a0 + P.b[OFF_B5 + 0];
-  o[1] = a1 + P.b[OFF_B5 + 1];
-  o[2] = a2 + P.b[OFF_B5 + 2];
 }
 
 // Input of keypoint (px, py): for level l in (la, lb), the 16 x 16 integer
