@@ -30,6 +30,35 @@ namespace det {
 constexpr int kHalo = 4;
 constexpr int kThreads = 128;   // CTA size of the standalone detection launches
 
+// Three-input and add-then-maximum instructions on 16-bit lanes (one
+// instruction each on this GPU).
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned min3_u16x2(unsigned a, unsigned b, unsigned c) {
+  return __vimin3_u16x2(a, b, c);
+}
+__device__ __forceinline__ unsigned max3_u16x2(unsigned a, unsigned b, unsigned c) {
+  return __vimax3_u16x2(a, b, c);
+}
+__device__ __forceinline__ unsigned addmax_s16x2(unsigned a, unsigned b, unsigned c) {
+  return __viaddmax_s16x2(a, b, c);
+}
+#else
+inline unsigned min3_u16x2(unsigned a, unsigned b, unsigned c) {
+  return __vminu2(__vminu2(a, b), c);
+}
+inline unsigned max3_u16x2(unsigned a, unsigned b, unsigned c) {
+  return __vmaxu2(__vmaxu2(a, b), c);
+}
+inline unsigned addmax_s16x2(unsigned a, unsigned b, unsigned c) {
+  unsigned r = 0;
+  for (int s = 0; s < 32; s += 16) {
+    const int v = (int16_t)(uint16_t)((a >> s) + (b >> s)), w = (int16_t)(uint16_t)(c >> s);
+    r |= (unsigned)(uint16_t)(v > w ? v : w) << s;
+  }
+  return r;
+}
+#endif
+
 // score + 1 in [0, 255], 0 = no corner at tau >= 0
 __device__ __forceinline__ int fast_m(const int v[16], int c) {
   int p_lo[16], p_hi[16];
@@ -72,25 +101,21 @@ __device__ __forceinline__ int ring_dy(int k) {
 // A CTA of NT threads takes a block of bcx x bcy cells, g warps per cell
 // (g * bcx * bcy <= NT / 32; g = 1 when there are many cells to fill the GPU
 // with, more when a launch has few cells), and stages the block's level-0
-// region with its halo once, widened to 16 bits: every 32-bit shared word
-// holds two horizontally adjacent pixels, so the bound, the masks and the
-// threshold windows run on two pixels per instruction (16x2 min/max are
-// native on this GPU, byte-wise SIMD is not); each thread takes four pixels
-// (two words) at a time.
+// region with its halo once. The bound runs on 16-bit lanes, two pixels per
+// instruction (16x2 min/max are native on this GPU, byte-wise SIMD is not);
+// each thread takes four pixels (a 32-bit word) at a time.
 //
-// Per cell the group keeps one map over the cell and its 1-pixel ring, 16 bits
-// per pixel: high byte = ub - T_min, low byte = (m - T_min) where the exact
-// score m is known, the bound ub elsewhere, both clamped at 0 (0 = cannot be
-// a candidate). The shift by T_min keeps every comparison of the algorithm
+// Values carry a shift by T_min, clamped at 0: ub - T_min of the bound, m -
+// T_min of the exact score m. The shift keeps every comparison of the algorithm
 // (thresholds, strict maxima) and leaves 0 for "no corner >= T_min".
 //
 // Exact branch-and-bound. A 9-arc holds one pixel of each opposite pair
 // (0,8) and (4,12) (the paper's early rejection), so with m = score + 1,
 //   m <= ub = max(min(max(v0,v8), max(v4,v12)) - c, c - max(min(v0,v8), min(v4,v12))).
 // Exact scores are computed only for pixels whose bound reaches a threshold
-// t, which starts 24 below the largest bound of the cell and its ring and is
-// lowered in steps of 24 until at least k candidates with m >= t are known
-// (or t reaches T_min + 1). After every pixel with ub >= t is evaluated, every
+// t, which starts at a share of the largest bound of the cell and its ring and
+// is lowered until at least k candidates with m >= t are known (or t reaches
+// T_min + 1). After every pixel with ub >= t is evaluated, every
 // pixel with m >= t has its 3x3 maximum test decided: a neighbour either is
 // evaluated (exact comparison) or has ub < t <= m. So the candidates with
 // m >= t are exactly known, and if there are k of them no other pixel can
@@ -100,10 +125,11 @@ __device__ __forceinline__ int ring_dy(int k) {
 struct BlockSmem {
   int rs, rows, stage_bytes;  // staged region: row stride (bytes), rows, bytes
   int msb, mh;                // maps: row stride (bytes, multiple of 8), rows
+  int map_bytes;              // a map, whole 16-byte words
   int g;                      // warps per cell
-  int qcap, kcap;             // queue and key entries per warp
+  int qcap, scap, kcap;       // queue, scored-list and key entries per warp
   int c_u, c_v, c_cols, c_red, c_merge, per_cell;  // byte offsets in a cell's piece
-  int w_queue, w_keys, per_warp;                   // byte offsets in a warp's piece
+  int w_queue, w_scored, w_keys, per_warp;         // byte offsets in a warp's piece
   int cells_bytes, total;
 };
 
@@ -121,16 +147,19 @@ __host__ __device__ inline BlockSmem block_smem(int cw, int ch, int k, int bcx, 
   S.msb = (cw + 5 + 7) & ~7;
   S.mh = ch + 2;
   S.g = g;
-  S.qcap = 384;                                    // beyond it: pass C scans the map
+  S.qcap = 1024;                  // drained when a scan step (512 pixels) may not fit
+  S.scap = 384;                   // beyond it: pass C scans the map
   S.kcap = k + 32;
+  S.map_bytes = pyr::up16(S.msb * S.mh);
   S.c_u = 16;                                      // guards around both maps
-  S.c_v = S.c_u + pyr::up16(S.msb * S.mh) + 16;
-  S.c_cols = S.c_v + pyr::up16(S.msb * S.mh) + 16;
+  S.c_v = S.c_u + S.map_bytes + 16;
+  S.c_cols = S.c_v + S.map_bytes + 16;
   S.c_red = S.c_cols + 8 * (S.msb / 4);
   S.c_merge = S.c_red + pyr::up16(4 * 2 * g);
   S.per_cell = S.c_merge + pyr::up16(8 * g * k);
-  S.w_queue = 0;
-  S.w_keys = pyr::up16(2 * S.qcap);
+  S.w_queue = 16;                                  // after the queue's fill count
+  S.w_scored = S.w_queue + pyr::up16(2 * S.qcap);
+  S.w_keys = S.w_scored + pyr::up16(2 * S.scap);
   S.per_warp = S.w_keys + pyr::up16(8 * S.kcap);
   S.cells_bytes = bcx * bcy * S.per_cell;
   S.total = S.stage_bytes + S.cells_bytes + bcx * bcy * g * S.per_warp;
@@ -200,28 +229,42 @@ __device__ __forceinline__ unsigned bytes_ge(unsigned a, unsigned tb, unsigned t
 }
 
 // m = score + 1 of the pixel at q (staged bytes, row stride rs), 0 if none:
-// bright and dark arcs together, (v, 255 - v) in the two 16-bit lanes.
+// bright and dark arcs together, (v, 255 - v) in the two 16-bit lanes. The
+// minimum of nine ring pixels is that of three triples.
 __device__ __forceinline__ int fast_m_pair(const uint8_t* q, int rs) {
-  unsigned V[16];
+  unsigned V[16], T[16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const unsigned s = q[ring_dy(k) * rs + ring_dx(k)];
-    V[k] = s | ((255u - s) << 16);
-  }
-  unsigned P[16], Q[16];
+  for (int k = 0; k < 16; ++k)   // s + ((255 - s) << 16)
+    V[k] = (unsigned)q[ring_dy(k) * rs + ring_dx(k)] * 0xffff0001u + 0x00ff0000u;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) P[k] = __vminu2(V[k], V[(k + 1) & 15]);
-#pragma unroll
-  for (int k = 0; k < 16; ++k) Q[k] = __vminu2(P[k], P[(k + 2) & 15]);
-  // arc k..k+8 = quads k, k+4 and k+5 (overlapping: min is idempotent)
+  for (int k = 0; k < 16; ++k) T[k] = min3_u16x2(V[k], V[(k + 1) & 15], V[(k + 2) & 15]);
   unsigned best = 0;
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    best = __vmaxu2(best, __vminu2(__vminu2(Q[k], Q[(k + 4) & 15]), Q[(k + 5) & 15]));
+  for (int k = 0; k < 16; k += 2)
+    best = max3_u16x2(best, min3_u16x2(T[k], T[(k + 3) & 15], T[(k + 6) & 15]),
+                      min3_u16x2(T[k + 1], T[(k + 4) & 15], T[(k + 7) & 15]));
   const int c = q[0];
   const int lo = (int)(best & 0xffffu);          // max over arcs of the arc minimum
   const int hi = 255 - (int)(best >> 16);        // min over arcs of the arc maximum
   const int m = max(lo - c, c - hi);
+  return m > 0 ? m : 0;
+}
+
+// A bound of fast_m_pair from every other ring pixel: a 9-arc holds four
+// consecutive ones of these eight.
+__device__ __forceinline__ int bound8_pair(const uint8_t* q, int rs) {
+  unsigned V[8], P[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    V[k] = (unsigned)q[ring_dy(2 * k) * rs + ring_dx(2 * k)] * 0xffff0001u + 0x00ff0000u;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) P[k] = __vminu2(V[k], V[(k + 1) & 7]);
+  unsigned best = 0;
+#pragma unroll
+  for (int k = 0; k < 8; k += 2)
+    best = max3_u16x2(best, __vminu2(P[k], P[(k + 2) & 7]), __vminu2(P[k + 1], P[(k + 3) & 7]));
+  const int c = q[0];
+  const int m = max((int)(best & 0xffffu) - c, c - (255 - (int)(best >> 16)));
   return m > 0 ? m : 0;
 }
 
@@ -239,8 +282,10 @@ __device__ __forceinline__ int warp_top_keys(const unsigned long long* keys, int
   const int lane = threadIdx.x & 31;
   unsigned long long last = ~0ull;
   int got = 0;
+#pragma unroll 1
   for (int round = 0; round < k; ++round) {
     unsigned long long best = 0;
+#pragma unroll 1
     for (int e = lane; e < n; e += 32) {
       const unsigned long long key = keys[e];
       if (key < last && key > best) best = key;
@@ -263,6 +308,7 @@ struct CellGeom {
   int cw, ch, gx, k, tmin, border;
   int bcx, bcy, g;   // cells per CTA, warps per cell
   int sel;           // VIO_SELECT_* (per-cell top-k)
+  BlockSmem S;       // shared-memory layout of the launch (detect_setup)
 };
 
 // Bitonic sort of 64 keys, two per lane (element lane and lane + 32), into
@@ -337,19 +383,32 @@ __device__ __forceinline__ void group_sync(int g, int bar) {
   }
 }
 
-// Exact scores of queue entries [e0, e1) (one per lane) into the value map.
-__device__ __forceinline__ void eval_entries(const uint16_t* queue, int e0, int e1,
+// Exact scores of list entries [e0, e1) into the value map, 32 at a time.
+__device__ __forceinline__ void eval_entries(const uint16_t* list, int e0, int e1,
                                              const uint8_t* st, int rs, int srow0, int c0,
                                              const Split& sm, int T, uint8_t* vmap) {
-  const int e = e0 + (threadIdx.x & 31);
-  if (e < e1) {
-    const int idx = queue[e];
+#pragma unroll 1
+  for (int e = e0 + (int)(threadIdx.x & 31); e < e1; e += 32) {
+    const int idx = list[e];
     int r, c;
     sm(idx, r, c);
     const int m = fast_m_pair(st + (srow0 + r) * rs + c0 + c, rs);
     vmap[idx] = (uint8_t)max(m - T, 0);
   }
+  __syncwarp();
 }
+
+// n / 16 of threshold t (both shifted by -T). The first threshold is 10/16 of
+// the cell's largest bound for one keypoint per cell, 8/16 for more, the
+// second 11/16 of the first, each further one 6/16 of the one before. A
+// corner's score is about 0.6 of the largest bound of a textured cell, so one
+// round usually finds the strongest: over 300 cells of a 752 x 480 frame, 1.03
+// rounds, 136 bounds tightened and 50 pixels scored a cell (1.31 rounds and
+// 124 scored with steps of 24 from 24 below the largest bound and no second
+// bound). Where few corners are left (masks, several per cell) the steep tail
+// saves rounds: 12 masked images of 641 x 479, four per 50 x 50 cell, 118 us
+// against 142 us with 10/16 throughout.
+__device__ __forceinline__ int scaled(int t, int T, int n) { return (((t + T) * n) >> 4) - T; }
 
 // Detection in one cell by warp gw of its g warps. st: the block's staged
 // region (bytes, row stride rs, column 0 at image x sxa, a multiple of 16,
@@ -357,18 +416,27 @@ __device__ __forceinline__ void eval_entries(const uint16_t* queue, int e0, int 
 // count.
 //
 // Two byte maps cover the cell and its 1-pixel ring from a 4-pixel boundary
-// of the staged region (map column 0 at image x mx0), rows y0 - 1 .. y0 + ch:
-//   U: ub - T_min (clamped at 0), the bound; a pixel's byte is cleared once it
-//      is queued for its exact score, so each pixel is scored once;
-//   V: the value the 3x3 maximum test compares: (m - T_min)+ once scored, the
-//      bound before (a pixel that is not scored has ub < t <= m of any pixel
-//      tested against it).
+// of the staged region (map column 0 at image x mx0), rows y0 - 1 .. y0 + ch,
+// zero where nothing else is said:
+//   U: the bound ub - T_min, where the ring of the pixel lies in the image;
+//   V: m - T_min, once the pixel has been scored.
 // Pass A computes the bound four pixels per thread: the 32-bit staged word
 // x .. x + 3 splits into the 16-bit pairs (x, x + 2) and (x + 1, x + 3).
-// Each round at threshold t scans U eight pixels per thread with byte-wise
-// compares, queues the pixels whose bound reaches t and scores them 32 at a
-// time; pass C then tests every scored pixel with a value in [t, tp) for a
-// strict maximum in the cell.
+// Each round at threshold t (below the previous one, tp) scans U sixteen
+// pixels per thread with byte-wise compares and queues the pixels whose bound
+// lies in [t, tp). A queued pixel's bound is tightened first (eight ring
+// pixels; U keeps the result, so a pixel that falls below t waits for its
+// round) and what still reaches t is scored, 32 pixels at a time; pass C then
+// tests every scored pixel with a value in [t, tp) for a strict maximum in the
+// cell: a neighbour that has not been scored has m <= ub < t and holds 0.
+//
+// What bounds it: instructions, 2.7 thousand of a warp for a 37 x 32 cell (46%
+// staging, set-up and pass A, 16% the scan, 19% bounds and scores, the rest
+// tests, later rounds and the selection), issued at 62% of the rate; the loops
+// are not unrolled because the warps of an SM, each in another phase, miss in
+// the instruction cache. 185 images of 752 x 480: 294 us with a scan of eight
+// pixels a word, prefix sums for the queue and every queued pixel scored; 195
+// us so.
 template <bool MASKED>
 __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int rs, int sxa,
                                             int sy0, int W, int H, const CellGeom& cg, int cx,
@@ -384,47 +452,64 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
   const int x0 = cx * cw, y0 = cy * ch;
   const int c0 = (x0 - 1 - sxa) & ~3;                    // staged column of map column 0
   const int mx0 = sxa + c0;                              // image x of map column 0
-  const int MW = (x0 + cw + 1 - mx0 + 7) & ~7;           // map columns (multiple of 8)
-  const int nq = MW >> 2, n8 = MW >> 3;                  // quads, 8-pixel words per row
-  const int MH = ch + 2, MSB = S.msb;
+  const int nq = (x0 + cw + 1 - mx0 + 3) >> 2;           // quads per row that hold ring pixels
+  const int MSB = S.msb;
   const int srow0 = y0 - 1 - sy0;                        // staged row of map row 0
   uint8_t* umap = csm + S.c_u;
   uint8_t* vmap = csm + S.c_v;
   uint2* colm = reinterpret_cast<uint2*>(csm + S.c_cols);   // per quad: ring masks
   int* red = reinterpret_cast<int*>(csm + S.c_red);
   unsigned long long* merge = reinterpret_cast<unsigned long long*>(csm + S.c_merge);
+  volatile int* q_fill = reinterpret_cast<volatile int*>(wsm);
   uint16_t* queue = reinterpret_cast<uint16_t*>(wsm + S.w_queue);
+  uint16_t* scored = reinterpret_cast<uint16_t*>(wsm + S.w_scored);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsm + S.w_keys);
+  const int n16 = S.map_bytes >> 4;
 
-  // per quad: lanes where the bound is defined (FAST ring inside the image,
-  // inside the cell's ring region)
+  // zero maps; per quad: lanes where the bound is defined (FAST ring inside
+  // the image, inside the cell's ring region)
+#pragma unroll 1
+  for (int i = tg; i < n16; i += GT) {
+    reinterpret_cast<uint4*>(umap)[i] = make_uint4(0u, 0u, 0u, 0u);
+    reinterpret_cast<uint4*>(vmap)[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll 1
   for (int q = tg; q < nq; q += GT) {
     const int xq = mx0 + 4 * q;
     const int rl = max(x0 - 1, 3), rh = min(x0 + cw, W - 4);
     colm[q] = make_uint2(pair_mask2(xq, rl, rh), pair_mask2(xq + 1, rl, rh));
   }
+  if (lane == 0) *q_fill = 0;
   const bool atomic_sel = cg.sel == VIO_SELECT_ATOMIC;   // k == 1: one 64-bit maximum per cell
   if (atomic_sel && tg == 0) merge[0] = 0ull;
   group_sync(G, bar);
 
   // pass A: bounds of the cell and its ring and the largest of them (it only
   // sets the first threshold: any start at or above the largest bound of the
-  // cell's unmasked pixels gives the same result); this
-  // thread's quads i = tg + j * GT -> (row r, quad q), stepped without divisions
-  const unsigned K = (0x100u + (unsigned)T) * 0x00010001u;
+  // cell's unmasked pixels gives the same result), over the rows whose FAST
+  // ring lies in the image; this thread's quads i = tg + j * GT -> (row, quad
+  // q), stepped without divisions
+  const unsigned NK = (unsigned)(-(255 + T)) & 0xffffu, NK2 = NK | (NK << 16);
   unsigned acc = 0;
   {
-    const int n_items = MH * nq;
+    const int r_lo = max(0, 4 - y0), r_hi = min(ch + 2, H - 2 - y0);   // map rows
+    const int n_items = max(0, r_hi - r_lo) * nq;
     const int dr = GT / nq, dq = GT - dr * nq;
-    int r = tg / nq, q = tg - (tg / nq) * nq;
+    const int rr = tg / nq;
+    int q = tg - rr * nq;
+    const uint8_t* sq = st + (srow0 + r_lo + rr) * rs + c0 + 4 * q;   // pixels x .. x + 3
+    uint8_t* uq = umap + (r_lo + rr) * MSB + 4 * q;
+    const int rs3 = 3 * rs;
+    const int s_step = dr * rs + 4 * dq, u_step = dr * MSB + 4 * dq;
+    const int s_wrap = rs - 4 * nq, u_wrap = MSB - 4 * nq;
+#pragma unroll 2
     for (int i = tg; i < n_items; i += GT) {
-      const int y = y0 - 1 + r;
-      const uint8_t* sq = st + (srow0 + r) * rs + c0 + 4 * q;           // pixels x .. x + 3
       const unsigned Cw = *reinterpret_cast<const unsigned*>(sq);
-      const unsigned Uw = *reinterpret_cast<const unsigned*>(sq - 3 * rs);
-      const unsigned Dw = *reinterpret_cast<const unsigned*>(sq + 3 * rs);
+      const unsigned Uw = *reinterpret_cast<const unsigned*>(sq - rs3);
+      const unsigned Dw = *reinterpret_cast<const unsigned*>(sq + rs3);
       const unsigned Lw = *reinterpret_cast<const unsigned*>(sq - 4);
       const unsigned Rw = *reinterpret_cast<const unsigned*>(sq + 4);
+      const uint2 cm = colm[q];
       // pair a = pixels (x, x + 2), pair b = (x + 1, x + 3); compass points
       // of the ring: up, down (rows -3, +3), left (x - 3), right (x + 3)
       const unsigned Ca = __byte_perm(Cw, 0u, 0x4240), Cb = __byte_perm(Cw, 0u, 0x4341);
@@ -434,26 +519,25 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
       const unsigned Lb = __byte_perm(Lw, Cw, 0x0402) & 0x00ff00ffu;      // x - 2, x
       const unsigned Ra = __byte_perm(Cw, Rw, 0x0503) & 0x00ff00ffu;      // x + 3, x + 5
       const unsigned Rb = __byte_perm(Rw, 0u, 0x4240);                     // x + 4, x + 6
-      const unsigned hia = __vminu2(__vmaxu2(Ua, Da), __vmaxu2(Ra, La));
-      const unsigned loa = __vmaxu2(__vminu2(Ua, Da), __vminu2(Ra, La));
-      const unsigned hib = __vminu2(__vmaxu2(Ub, Db), __vmaxu2(Rb, Lb));
-      const unsigned lob = __vmaxu2(__vminu2(Ub, Db), __vminu2(Rb, Lb));
-      // 0x100 + max(hi - c, c - lo) per lane, then max(ub - T, 0)
-      const unsigned da = __vmaxu2(hia + 0x01000100u - Ca, Ca + 0x01000100u - loa);
-      const unsigned db = __vmaxu2(hib + 0x01000100u - Cb, Cb + 0x01000100u - lob);
-      const uint2 cm = colm[q];
-      const bool yf = y >= 3 && y <= H - 4;
-      const unsigned ua = (__vmaxu2(da, K) - K) & (yf ? cm.x : 0u);
-      const unsigned ub = (__vmaxu2(db, K) - K) & (yf ? cm.y : 0u);
-      const unsigned word = __byte_perm(ua, ub, 0x6240);                   // x .. x + 3
-      *reinterpret_cast<unsigned*>(umap + r * MSB + 4 * q) = word;
-      *reinterpret_cast<unsigned*>(vmap + r * MSB + 4 * q) = word;
-      acc = __vmaxu2(acc, __vmaxu2(ua, ub));
+      // max(hi - c, c - lo) + 255 per lane, with 255 - v as a complement, then
+      // max(ub - T, 0)
+      auto bound = [&](unsigned C, unsigned U, unsigned D, unsigned L, unsigned R) {
+        const unsigned hi = __vminu2(__vmaxu2(U, D), __vmaxu2(R, L));
+        const unsigned lo = __vmaxu2(__vminu2(U, D), __vminu2(R, L));
+        const unsigned up = hi + (C ^ 0x00ff00ffu);
+        return addmax_s16x2(addmax_s16x2(lo ^ 0x00ff00ffu, C, up), NK2, 0u);
+      };
+      const unsigned ua = bound(Ca, Ua, Da, La, Ra) & cm.x;
+      const unsigned ub = bound(Cb, Ub, Db, Lb, Rb) & cm.y;
+      *reinterpret_cast<unsigned*>(uq) = __byte_perm(ua, ub, 0x6240);     // x .. x + 3
+      acc = max3_u16x2(acc, ua, ub);
       q += dq;
-      r += dr;
+      sq += s_step;
+      uq += u_step;
       if (q >= nq) {
         q -= nq;
-        ++r;
+        sq += s_wrap;
+        uq += u_wrap;
       }
     }
   }
@@ -468,63 +552,87 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
 
   const Split sm(MSB);
   const unsigned lt_mask = (1u << lane) - 1u;
-  int nk = 0, q_end = 0, q_eval = 0, fw = 0;
-  bool overflow = false;   // the queue lost scored pixels
+  int nk = 0, s_end = 0, s_eval = 0, fw = 0;
+  bool overflow = false;   // the scored list lost pixels
   if (umax > 0) {
     int tp = 256;              // t_prev, above every shifted value
-    int t = max(umax - 24, 1);
-    const int n_words = MH * n8;
-    const int dr8 = GT / n8, dc8 = GT - dr8 * n8;
+    int t = max(scaled(umax, T, k == 1 ? 10 : 8), 1), down = 11;
+    // tightens the bounds of the queued pixels, 32 at a time, and scores
+    // those that still reach t
+    auto drain = [&](int n) {
+#pragma unroll 1
+      for (int e0 = 0; e0 < n; e0 += 32) {
+        const int e = e0 + lane;
+        int idx = 0;
+        bool keep = false;
+        if (e < n) {
+          idx = queue[e];
+          int r, c;
+          sm(idx, r, c);
+          const int v = max(bound8_pair(st + (srow0 + r) * rs + c0 + c, rs) - T, 0);
+          umap[idx] = (uint8_t)v;
+          keep = v >= t;
+        }
+        const unsigned bk = __ballot_sync(FULL, keep);
+        if (bk == 0) continue;
+        if (s_end + __popc(bk) > S.scap) {   // full: score what is pending, drop the list
+          eval_entries(scored, s_eval, s_end, st, rs, srow0, c0, sm, T, vmap);
+          s_end = s_eval = 0;
+          overflow = true;
+        }
+        if (keep) scored[s_end + __popc(bk & lt_mask)] = (uint16_t)idx;
+        s_end += __popc(bk);
+        __syncwarp();
+        if (s_end - s_eval >= 32) {
+          eval_entries(scored, s_eval, s_eval + 32, st, rs, srow0, c0, sm, T, vmap);
+          s_eval += 32;
+        }
+      }
+    };
     for (;;) {
-      // pass B: queue this warp's pixels whose bound reaches t (their U
-      // bytes are cleared), exact scores 32 at a time
+      // pass B: queue this warp's pixels whose bound lies in [t, tp)
       {
         const unsigned tb = (unsigned)t * 0x01010101u, tlo = tb & 0x7f7f7f7fu;
-        int r = tg / n8, c8 = tg - (tg / n8) * n8;
-        for (int base = gw * 32; base < n_words; base += GT) {
+        const unsigned pb = (unsigned)tp * 0x01010101u, plo = pb & 0x7f7f7f7fu;
+        int fill = 0;
+#pragma unroll 1
+        for (int base = gw * 32; base < n16; base += GT) {
           const int i = base + lane;
-          uint2 w = make_uint2(0u, 0u);
-          const int idx0 = r * MSB + 8 * c8;
-          if (i < n_words) w = *reinterpret_cast<const uint2*>(umap + idx0);
-          c8 += dc8;
-          r += dr8;
-          if (c8 >= n8) {
-            c8 -= n8;
-            ++r;
+          uint4 w = make_uint4(0u, 0u, 0u, 0u);
+          if (i < n16) w = reinterpret_cast<const uint4*>(umap)[i];
+          unsigned h[4] = {bytes_ge(w.x, tb, tlo), bytes_ge(w.y, tb, tlo), bytes_ge(w.z, tb, tlo),
+                           bytes_ge(w.w, tb, tlo)};
+          if (tp < 256) {   // scored in an earlier round
+            h[0] &= ~bytes_ge(w.x, pb, plo);
+            h[1] &= ~bytes_ge(w.y, pb, plo);
+            h[2] &= ~bytes_ge(w.z, pb, plo);
+            h[3] &= ~bytes_ge(w.w, pb, plo);
           }
-          const unsigned hx = bytes_ge(w.x, tb, tlo), hy = bytes_ge(w.y, tb, tlo);
-          const int cnt = __popc(hx) + __popc(hy);
-          if (__ballot_sync(FULL, cnt != 0) == 0) continue;
-          int incl = cnt;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += v;
+          // bit 7 of byte b of word j -> bit 8 b + j
+          unsigned m = (h[0] >> 7) | (h[1] >> 6) | (h[2] >> 5) | (h[3] >> 4);
+          if (__ballot_sync(FULL, m != 0u) == 0) continue;
+          const int cnt = __popc(m);
+          int off = cnt ? atomicAdd(const_cast<int*>(q_fill), cnt) : 0;
+#pragma unroll 1
+          for (; m; m &= m - 1) {
+            const int e = __ffs(m) - 1;
+            queue[off++] = (uint16_t)(16 * i + 4 * (e & 3) + (e >> 3));
           }
-          const int total = __shfl_sync(FULL, incl, 31);
-          if (q_end + total > S.qcap) {   // full: score what is pending, drop the list
-            eval_entries(queue, q_eval, q_end, st, rs, srow0, c0, sm, T, vmap);
-            __syncwarp();
-            q_end = q_eval = 0;
-            overflow = true;
-          }
-          if (cnt) {
-            int off = q_end + incl - cnt;
-            for (unsigned h = hx; h; h &= h - 1) queue[off++] = (uint16_t)(idx0 + ((__ffs(h) - 1) >> 3));
-            for (unsigned h = hy; h; h &= h - 1) queue[off++] = (uint16_t)(idx0 + 4 + ((__ffs(h) - 1) >> 3));
-            w.x &= ~((hx >> 7) * 0xffu);
-            w.y &= ~((hy >> 7) * 0xffu);
-            *reinterpret_cast<uint2*>(umap + idx0) = w;
-          }
-          q_end += total;
           __syncwarp();
-          while (q_end - q_eval >= 32) {
-            eval_entries(queue, q_eval, q_eval + 32, st, rs, srow0, c0, sm, T, vmap);
-            q_eval += 32;
+          fill = *q_fill;
+          if (fill > S.qcap - 512) {   // another step may not fit
+            drain(fill);
+            __syncwarp();
+            if (lane == 0) *q_fill = 0;
+            __syncwarp();
+            fill = 0;
           }
         }
-        eval_entries(queue, q_eval, q_end, st, rs, srow0, c0, sm, T, vmap);
-        q_eval = q_end;
+        drain(fill);
+        __syncwarp();
+        if (lane == 0) *q_fill = 0;
+        eval_entries(scored, s_eval, s_end, st, rs, srow0, c0, sm, T, vmap);
+        s_eval = s_end;
       }
       group_sync(G, bar);
       // pass C: scored pixels with a value in [t, tp) that lie in the cell
@@ -570,24 +678,17 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
         __syncwarp();
       };
       if (!overflow) {
-        for (int base = 0; base < q_end; base += 32) {
+#pragma unroll 1
+        for (int base = 0; base < s_end; base += 32) {
           const int e = base + lane;
-          consider(e < q_end ? test(queue[e]) : 0ull);
+          consider(e < s_end ? test(scored[e]) : 0ull);
         }
       } else {
-        // the 8-pixel words this warp scanned in pass B (the pixels it queued)
-        int r = tg / n8, c8 = tg - (tg / n8) * n8;
-        for (int base = gw * 32; base < n_words; base += GT) {
-          const bool live = base + lane < n_words;
-          const int idx0 = r * MSB + 8 * c8;
-          c8 += dc8;
-          r += dr8;
-          if (c8 >= n8) {
-            c8 -= n8;
-            ++r;
-          }
+        // the 16-pixel words this warp scanned in pass B
+        for (int base = gw * 32; base < n16; base += GT) {
+          const int i = base + lane;
 #pragma unroll 1
-          for (int j = 0; j < 8; ++j) consider(live ? test(idx0 + j) : 0ull);
+          for (int j = 0; j < 16; ++j) consider(i < n16 ? test(16 * i + j) : 0ull);
         }
       }
       // candidates of the whole cell (all g warps, all rounds so far)
@@ -601,7 +702,8 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
       }
       if (n_found >= k || t <= 1) break;
       tp = t;
-      t = max(t - 24, 1);
+      t = max(scaled(t, T, down), 1);
+      down = 6;
     }
   }
   // top k of the cell: each warp's best k, then the best k of those (or,
@@ -643,8 +745,10 @@ __device__ __forceinline__ void detect_block(const uint8_t* __restrict__ src, in
   const int ncx = min(cg.bcx, cg.gx - c0x), ncy = min(cg.bcy, gy - c0y);
   const int bx0 = c0x * cg.cw, bx1 = (c0x + ncx) * cg.cw;
   const int by0 = c0y * cg.ch, by1 = (c0y + ncy) * cg.ch;
-  const BlockSmem S = block_smem(cg.cw, cg.ch, cg.k, cg.bcx, cg.bcy, cg.g);
-  pyr::stage_rect(src, W, H, P, bx0 - 8, bx1 + 12, by0 - kHalo, by1 + kHalo, smem, S.rs);
+  const BlockSmem& S = cg.S;
+  // pixels outside the image are never used: the bound and the scores read
+  // only rings that lie inside it
+  pyr::stage_rect<false>(src, W, H, P, bx0 - 8, bx1 + 12, by0 - kHalo, by1 + kHalo, smem, S.rs);
   __syncthreads();
   const int warp = threadIdx.x >> 5;
   const int ci = warp / cg.g, gw = warp - ci * cg.g;
@@ -661,7 +765,8 @@ __device__ __forceinline__ void detect_block(const uint8_t* __restrict__ src, in
 // per cell; returns the dynamic shared memory, or -1.
 inline int detect_setup(CellGeom& cg, int nt, int g_want) {
   if (!pick_block(cg.cw, cg.ch, cg.k, nt, g_want, cg.bcx, cg.bcy, cg.g)) return -1;
-  return block_smem(cg.cw, cg.ch, cg.k, cg.bcx, cg.bcy, cg.g).total;
+  cg.S = block_smem(cg.cw, cg.ch, cg.k, cg.bcx, cg.bcy, cg.g);
+  return cg.S.total;
 }
 
 }  // namespace det

@@ -133,11 +133,39 @@ __host__ __device__ inline PassPlan pass_plan(const int* wl, const int* hl, int 
   return P;
 }
 
-// Stages the clamped rectangle [x0, x1) x [y0, y1) of a w x h image into
-// shared memory: row r at dst + r * dstride, column j <-> x = (x0 & ~15) + j.
-// Interior 16-byte chunks are single vector loads when the image base and
-// pitch allow it; chunks touching the image edge load byte by byte with
-// replicated (clamped) coordinates.
+// 16 pixels at p inside a row of an image that ends at `end` (and starts before
+// p), p on any byte: five aligned words shifted into place. A word that would
+// reach past the image is put together from bytes.
+__device__ __forceinline__ uint4 load16_any(const uint8_t* __restrict__ p,
+                                            const uint8_t* __restrict__ begin,
+                                            const uint8_t* __restrict__ end) {
+  const unsigned o = (unsigned)(reinterpret_cast<uintptr_t>(p) & 3);
+  const uint8_t* q = p - o;
+  unsigned w[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const uint8_t* a = q + 4 * k;
+    w[k] = 0u;
+    if (a >= begin && a + 4 <= end) {
+      w[k] = __ldg(reinterpret_cast<const unsigned*>(a));
+    } else {
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (a + b >= begin && a + b < end) w[k] |= (unsigned)__ldg(a + b) << (8 * b);
+    }
+  }
+  return make_uint4(__funnelshift_r(w[0], w[1], 8 * o), __funnelshift_r(w[1], w[2], 8 * o),
+                    __funnelshift_r(w[2], w[3], 8 * o), __funnelshift_r(w[3], w[4], 8 * o));
+}
+
+// Stages the rectangle [x0, x1) x [y0, y1) of a w x h image into shared memory:
+// row r at dst + r * dstride, column j <-> x = (x0 & ~15) + j, in 16-byte
+// chunks: single vector loads when the image base and pitch allow it, else
+// words shifted into place (load16_any). CLAMP: pixels outside the image are
+// copies of its edge (chunks that touch the image edge load byte by byte);
+// else they are left as they are, and rows and chunks that lie outside whole
+// cost nothing.
+template <bool CLAMP = true>
 __device__ __forceinline__ void stage_rect(const uint8_t* __restrict__ img, int w, int h,
                                            int pitch, int x0, int x1, int y0, int y1,
                                            uint8_t* dst, int dstride) {
@@ -145,6 +173,7 @@ __device__ __forceinline__ void stage_rect(const uint8_t* __restrict__ img, int 
   const int nc = (x1 - xa + 15) >> 4;
   const int rows = y1 - y0;
   const bool vec_ok = ((reinterpret_cast<uintptr_t>(img) | (uintptr_t)pitch) & 15) == 0;
+  const uint8_t* end = img + (long long)(h - 1) * pitch + w;
   const int nt = blockDim.x;
   // each thread keeps one chunk column and steps over rows (rpi rows per
   // step over the block), four rows in flight
@@ -155,29 +184,42 @@ __device__ __forceinline__ void stage_rect(const uint8_t* __restrict__ img, int 
   for (int cc = c; cc < nc; cc += (rpi > 0 ? nc : nt)) {
     if (r0 >= rstep) break;
     const int gx = xa + 16 * cc;
-    const bool fast = vec_ok && gx >= 0 && gx + 16 <= w;
+    if (!CLAMP && (gx + 16 <= 0 || gx >= w)) continue;
+    // a chunk that starts inside the image ends inside the pitch when rows
+    // are 16-byte aligned
+    const bool in = gx >= 0 && (gx + 16 <= w || (!CLAMP && vec_ok));
     uint8_t* d0 = dst + 16 * cc;
-    for (int r = r0; r < rows; r += 4 * rstep) {
-      uint4 v[4];
+    if (in && vec_ok) {
+      for (int r = r0; r < rows; r += 4 * rstep) {
+        uint4 v[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int rr = r + u * rstep;
-        if (fast && rr < rows)
-          v[u] = __ldg(reinterpret_cast<const uint4*>(
-              img + (long long)clampi(y0 + rr, 0, h - 1) * pitch + gx));
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int rr = r + u * rstep;
-        if (rr >= rows) continue;
-        uint8_t* d = d0 + rr * dstride;
-        if (fast) {
-          *reinterpret_cast<uint4*>(d) = v[u];
-        } else {
-          const uint8_t* row = img + (long long)clampi(y0 + rr, 0, h - 1) * pitch;
-#pragma unroll
-          for (int b = 0; b < 16; ++b) d[b] = __ldg(row + clampi(gx + b, 0, w - 1));
+        for (int u = 0; u < 4; ++u) {
+          const int rr = r + u * rstep, y = y0 + rr;
+          if (rr < rows && (CLAMP || (y >= 0 && y < h)))
+            v[u] = __ldg(reinterpret_cast<const uint4*>(
+                img + (long long)(CLAMP ? clampi(y, 0, h - 1) : y) * pitch + gx));
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int rr = r + u * rstep, y = y0 + rr;
+          if (rr < rows && (CLAMP || (y >= 0 && y < h)))
+            *reinterpret_cast<uint4*>(d0 + rr * dstride) = v[u];
+        }
+      }
+      continue;
+    }
+#pragma unroll 1
+    for (int rr = r0; rr < rows; rr += rstep) {
+      const int y = y0 + rr;
+      if (!CLAMP && (y < 0 || y >= h)) continue;
+      const uint8_t* row = img + (long long)clampi(y, 0, h - 1) * pitch;
+      uint8_t* d = d0 + rr * dstride;
+      if (in) {
+        *reinterpret_cast<uint4*>(d) = load16_any(row + gx, img, end);
+      } else {
+#pragma unroll 4
+        for (int b = 0; b < 16; ++b)
+          if (CLAMP || (gx + b >= 0 && gx + b < w)) d[b] = __ldg(row + clampi(gx + b, 0, w - 1));
       }
     }
   }
