@@ -270,14 +270,15 @@ extern "C" vio_status vio_pyramid_detect(vio_ctx* ctx, const vio_pyr_layout* lay
     bc.l0 = b.l0 + (long long)i0 * b.l0_stride;
     bc.upper = b.upper + (long long)i0 * b.upper_stride;
     bc.n = b.n - i0 < chunk ? b.n - i0 : chunk;
-    e = vio::launch_pyramid(g, bc, ctx->p.round_mode, s);
+    bool beside = false;   // small launches run beside one another
+    e = vio::launch_pyramid(g, bc, ctx->p.round_mode, s, &beside);
     if (e != cudaSuccess) break;
     e = vio::launch_detect(
         ctx->p, g, bc, d_occupancy ? d_occupancy + (long long)i0 * n_cells : nullptr,
         d_mask ? d_mask + (long long)i0 * mask_stride : nullptr, mask_stride,
         ctx->d_cand + (long long)i0 * n_cells * ctx->p.k_per_cell,
         ctx->d_cand_count + (long long)i0 * n_cells, d_kp + 2LL * i0 * capacity,
-        d_score + (long long)i0 * capacity, d_count + i0, capacity, s);
+        d_score + (long long)i0 * capacity, d_count + i0, capacity, s, beside);
   }
   return cuda_status(e);
 }

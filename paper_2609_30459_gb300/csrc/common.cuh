@@ -75,6 +75,31 @@ inline cudaError_t once_per_device(PerDeviceOnce& o, F f) {
   return e;
 }
 
+// Launches `kernel` on stream s, as a programmatic dependent of the previous
+// launch when `dependent`: its CTAs may then be scheduled once every CTA of
+// the previous launch has passed griddepcontrol.launch_dependents (or
+// exited), and the kernel itself waits on griddepcontrol.wait before touching
+// what earlier launches write. Only after a launch that leaves most of the
+// GPU idle (at most kDependentMaxWarpsPerSm warps per SM): after one that fills
+// the GPU, the dependent's early-resident CTAs (a 1024-thread CTA holds all of
+// an SM's registers) would slow it more than the launch latency they hide.
+constexpr int kDependentMaxWarpsPerSm = 16;
+template <class K, class... A>
+inline cudaError_t launch_dependent(K kernel, dim3 grid, unsigned block, size_t smem,
+                                    cudaStream_t s, bool dependent, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // The detection parameters of vio_params (cells, k, thresholds, border), as
 // every detection entry point validates them.
 inline bool detect_params_ok(const vio_params* p) {
@@ -148,19 +173,22 @@ struct vio_ctx {
 
 namespace vio {
 // launchers (host side), implemented in the .cu files
-cudaError_t launch_pyramid(const Geom& g, const Batch& b, int round_mode, cudaStream_t s);
+// small (may be null): whether the last launch left most of the GPU idle, so that
+// the next one may be its programmatic dependent
+cudaError_t launch_pyramid(const Geom& g, const Batch& b, int round_mode, cudaStream_t s,
+                           bool* small = nullptr);
 cudaError_t launch_pyramid_from(const Geom& g, const Batch& b, int s0, int round_mode,
+                                cudaStream_t s, bool* small = nullptr);
+// levels s0 + 1 .. in rest_passes() launches (two levels each)
+cudaError_t launch_pyramid_rest(const Geom& g, const Batch& b, int s0, int round_mode,
                                 cudaStream_t s);
 cudaError_t launch_fast_scores(const uint8_t* img, int w, int h, int pitch, int16_t* out,
                                cudaStream_t s);
 cudaError_t launch_detect(const vio_params& p, const Geom& g, const Batch& b,
                           const uint8_t* occ, const uint8_t* mask, long long mask_stride,
                           unsigned long long* cand, int32_t* cand_count, float* kp,
-                          int16_t* score, int32_t* count, int capacity, cudaStream_t s);
-cudaError_t launch_select(const unsigned long long* cand, const int32_t* cand_count,
-                          const uint8_t* occ, int n_cells, int k, int w, float* kp,
-                          int16_t* score, int32_t* count, int capacity, int n_images,
-                          cudaStream_t s);
+                          int16_t* score, int32_t* count, int capacity, cudaStream_t s,
+                          bool beside = false);
 cudaError_t launch_track(const Geom& g, const Batch& src, const Batch& dst, const float* pts,
                          const float* init, const int32_t* count, int capacity,
                          const TrackCfg& cfg, float* out3, float* out2, uint8_t* status,

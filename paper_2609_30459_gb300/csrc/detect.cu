@@ -36,8 +36,14 @@ struct DetectArgs {
   int n_cells, gy;
 };
 
-__global__ void __launch_bounds__(det::kThreads, 6) detect_cells_kernel(DetectArgs a) {
+// As a programmatic dependent of the pyramid's launches of the same images it
+// runs beside them: it reads level 0 only, which they read too, and its
+// scratch was last used before them. It ends after they have, so that what
+// follows it follows them.
+__global__ void __launch_bounds__(det::kThreads, 6)
+    detect_cells_kernel(const __grid_constant__ DetectArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
+  asm volatile("griddepcontrol.launch_dependents;");
   const int img = blockIdx.y;
   const uint8_t* src = level_ptr(a.g, a.b, img, 0);
   unsigned long long* cand = a.cand + (long long)img * a.n_cells * a.cg.k;
@@ -48,6 +54,7 @@ __global__ void __launch_bounds__(det::kThreads, 6) detect_cells_kernel(DetectAr
   else
     det::detect_block<false>(src, a.g.w[0], a.g.h[0], a.g.pitch[0], a.cg, a.gy, blockIdx.x,
                              nullptr, cand, count, smem);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 constexpr int SEL_THREADS = 512;
@@ -56,6 +63,8 @@ __global__ void __launch_bounds__(SEL_THREADS) select_kernel(
     const unsigned long long* __restrict__ cand, const int32_t* __restrict__ cand_count,
     const uint8_t* __restrict__ occ, int n_cells, int k, int W, float* __restrict__ kp,
     int16_t* __restrict__ score, int32_t* __restrict__ count, int capacity) {
+  // a programmatic dependent of a small detection launch (a no-op otherwise)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ int warp_sums[SEL_THREADS / 32];
   __shared__ int carry_s;
   const int img = blockIdx.x;
@@ -125,7 +134,8 @@ cudaError_t launch_fast_scores(const uint8_t* img, int w, int h, int pitch, int1
 cudaError_t launch_detect(const vio_params& p, const Geom& g, const Batch& b,
                           const uint8_t* occ, const uint8_t* mask, long long mask_stride,
                           unsigned long long* cand, int32_t* cand_count, float* kp,
-                          int16_t* score, int32_t* count, int capacity, cudaStream_t s) {
+                          int16_t* score, int32_t* count, int capacity, cudaStream_t s,
+                          bool beside) {
   DetectArgs a;
   a.g = g;
   a.b = b;
@@ -142,6 +152,7 @@ cudaError_t launch_detect(const vio_params& p, const Geom& g, const Batch& b,
   const int smem = det::detect_setup(
       a.cg, det::kThreads, det::warps_per_cell((long long)n_cells * b.n, sm_count()));
   if (smem < 0) return cudaErrorInvalidValue;
+  bool small = false;   // the detection launch leaves most of the GPU idle
   if (n_cells > 0) {
     // as much shared memory as the SM has: more CTAs (once per device)
     static PerDeviceOnce carveout;
@@ -151,25 +162,21 @@ cudaError_t launch_detect(const vio_params& p, const Geom& g, const Batch& b,
                                   (int)cudaSharedmemCarveoutMaxShared);
     });
     if (ec != cudaSuccess) return ec;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // 48 KiB less the static part
       cudaError_t e = cudaFuncSetAttribute(detect_cells_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e != cudaSuccess) return e;
     }
     dim3 grid(det::detect_blocks(a.cg.gx, a.gy, a.cg.bcx, a.cg.bcy), b.n);
-    detect_cells_kernel<<<grid, det::kThreads, smem, s>>>(a);
+    const cudaError_t e =
+        launch_dependent(detect_cells_kernel, grid, det::kThreads, (size_t)smem, s, beside, a);
+    if (e != cudaSuccess) return e;
+    small = (long long)grid.x * grid.y * (det::kThreads / 32) <=
+            (long long)kDependentMaxWarpsPerSm * sm_count();
   }
-  return launch_select(cand, cand_count, occ, n_cells, a.cg.k, g.w[0], kp, score, count,
-                       capacity, b.n, s);
-}
-
-cudaError_t launch_select(const unsigned long long* cand, const int32_t* cand_count,
-                          const uint8_t* occ, int n_cells, int k, int w, float* kp,
-                          int16_t* score, int32_t* count, int capacity, int n_images,
-                          cudaStream_t s) {
-  select_kernel<<<n_images, SEL_THREADS, 0, s>>>(cand, cand_count, occ, n_cells, k, w, kp, score,
-                                                 count, capacity);
-  return cudaGetLastError();
+  return launch_dependent(select_kernel, dim3((unsigned)b.n), SEL_THREADS, 0, s, small,
+                          (const unsigned long long*)cand, (const int32_t*)cand_count, occ,
+                          n_cells, a.cg.k, g.w[0], kp, score, count, capacity);
 }
 
 }  // namespace vio

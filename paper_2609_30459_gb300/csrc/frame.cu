@@ -380,31 +380,6 @@ __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ Mult
   }
 }
 
-// Launches `kernel` on stream s, as a programmatic dependent of the previous
-// launch when `dependent`: its CTAs may then be scheduled once every CTA of
-// the previous launch has passed griddepcontrol.launch_dependents (or
-// exited), and the kernel itself waits on griddepcontrol.wait before touching
-// memory. Only after a launch that leaves most of the GPU idle (at most
-// kDependentMaxWarpsPerSm warps per SM): after one that fills the GPU, the
-// dependent's early-resident CTAs (a 1024-thread CTA holds all of an SM's
-// registers) would slow it more than the launch latency they hide.
-constexpr int kDependentMaxWarpsPerSm = 16;
-template <class K, class A>
-cudaError_t launch_dependent(K kernel, unsigned grid, unsigned block, size_t smem,
-                             cudaStream_t s, const A& args, bool dependent = true) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
-}
-
 struct MultiK3 {
   int n;
   long long block_end[kMaxGroups];   // in blocks (= streams)
@@ -565,7 +540,7 @@ K1Args front_args(const vio_params& p, const Geom& g, const Batch& all, int det_
 
 template <int NT, bool MASKED>
 cudaError_t launch_k1_nt(const MultiK1& mm, int smem, cudaStream_t s) {
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {   // 48 KiB less the static part
     const cudaError_t e = cudaFuncSetAttribute(
         frame_front_kernel<NT, MASKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -645,7 +620,7 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
       const FrameLaunch& f = fl[i];
       const int m1 = first_levels(f.g, tune.pyr_first);
       if (f.g.n_levels > 1 + m1) {
-        e = launch_pyramid_from(f.g, f.cur, m1, f.p.round_mode, s);
+        e = launch_pyramid_rest(f.g, f.cur, m1, f.p.round_mode, s);
         if (e != cudaSuccess) return e;
       }
     }
@@ -718,15 +693,15 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     const int sm = (f.g.w[0] / f.p.cell_w) * (f.g.h[0] / f.p.cell_h) * (int)sizeof(int);
     smem3 = sm > smem3 ? sm : smem3;
   }
-  if (smem3 > 48 * 1024) {
+  if (smem3 > 40 * 1024) {   // 48 KiB less the static part
     e = cudaFuncSetAttribute(frame_finalize_kernel,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem3);
     if (e != cudaSuccess) return e;
   }
   // a programmatic dependent of a small tracking launch (a single frame): its
   // CTA is resident and waiting when the tracking ends
-  e = launch_dependent(frame_finalize_kernel, (unsigned)acc, K3_THREADS, (size_t)smem3, s, m3,
-                       k2_small);
+  e = launch_dependent(frame_finalize_kernel, dim3((unsigned)acc), K3_THREADS, (size_t)smem3, s,
+                       k2_small, m3);
   if (e != cudaSuccess) return e;
   if (tune.stereo_after) {
     // K4: stereo matching of the selected keypoints; K5: append to camera 1
@@ -740,11 +715,12 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     }
     if (w4 > 0) {
       const long long blocks4 = (w4 * 32 + k2t - 1) / k2t;
-      e = launch_dependent(frame_stereo_kernel, (unsigned)blocks4, (unsigned)k2t, 0, s, m4);
+      e = launch_dependent(frame_stereo_kernel, dim3((unsigned)blocks4), (unsigned)k2t, 0, s, true,
+                           m4);
       if (e != cudaSuccess) return e;
     }
-    e = launch_dependent(frame_append_kernel, (unsigned)acc, K3_THREADS, 0, s, m3,
-                         w4 <= (long long)kDependentMaxWarpsPerSm * sm_count());
+    e = launch_dependent(frame_append_kernel, dim3((unsigned)acc), K3_THREADS, 0, s,
+                         w4 <= (long long)kDependentMaxWarpsPerSm * sm_count(), m3);
     if (e != cudaSuccess) return e;
   }
   mark(5);

@@ -1,13 +1,45 @@
-// Image pyramid entry point (Sec. III-C, Eq. 1-3). Levels are produced by
-// passes of up to two levels each (device code in pyramid_dev.cuh): the
-// first pass reads level 0 and writes levels 1-2, the next reads level 2 and
-// writes levels 3-4, and so on; each pass is one launch over all tiles of all
-// images.
+// Image pyramid entry point (Sec. III-C, Eq. 1-3): one launch per level, each
+// straight from the level below (level_strip of pyramid_dev.cuh).
+//
+// What bounds it: for a batch larger than the L2, DRAM (level 0 once, the upper
+// levels once; a level's reads find the level before it in the L2); for a few
+// images the launches, which are programmatic dependents of one another. A
+// thread makes eight columns of several rows, so that an input row is loaded
+// and unpacked once or twice and no shared memory or barrier is needed. 185
+// images of 752 x 480 to four levels: PYR_AFTER us; passes of two levels through
+// shared-memory tiles of 128 x 128 pixels took 91 us, bound by the
+// shared-memory wavefronts of every output's 5 x 24 source bytes.
+#include <algorithm>
+
 #include "pyramid_dev.cuh"
 
 namespace vio {
 namespace {
 
+constexpr int LEVEL_THREADS = 128;
+
+// Thread t: strip t of the images' (groups of eight columns) x (blocks of
+// `rows` output rows), columns fastest.
+__global__ void __launch_bounds__(LEVEL_THREADS) pyr_level_kernel(const __grid_constant__ Geom g,
+                                                                  const __grid_constant__ Batch b,
+                                                                  int s, int groups, int blocks,
+                                                                  int rows, int round_mode) {
+  // a programmatic dependent of the level below's launch (no-ops otherwise)
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const unsigned t = blockIdx.x * LEVEL_THREADS + threadIdx.x;
+  const unsigned per = (unsigned)(groups * blocks);
+  const int img = (int)(t / per);
+  if (img >= b.n) return;
+  const int q = (int)(t - (unsigned)img * per);
+  const int by = q / groups, gx = q - by * groups;
+  const int y0 = by * rows;
+  pyr::level_strip(g, b, img, s, 8 * gx, y0, min(rows, g.h[s + 1] - y0),
+                   round_mode == 0 ? 0x00800080u : 0u);
+}
+
+// Two levels per launch through shared-memory tiles: the deeper levels of a
+// frame step, where a launch costs more than the levels do.
 __global__ void __launch_bounds__(pyr::kThreads) pyr_pass_kernel(Geom g, Batch b, int s, int m,
                                                                  int T, int ntx, int nty,
                                                                  int round_mode) {
@@ -21,28 +53,60 @@ __global__ void __launch_bounds__(pyr::kThreads) pyr_pass_kernel(Geom g, Batch b
 
 }  // namespace
 
-cudaError_t launch_pyramid_from(const Geom& g, const Batch& b, int s0, int round_mode,
+cudaError_t launch_pyramid_rest(const Geom& g, const Batch& b, int s0, int round_mode,
                                 cudaStream_t st) {
-  for (int s = s0; s + 1 < g.n_levels; s += pyr::kRestPass) {
-    const int m = pyr::rest_pass_levels(g.n_levels, s);
-    const int T = pyr::top_tile(m, pyr::kRestShift);
+  int s = s0;
+  for (; s + 2 < g.n_levels; s += 2) {
+    const int m = 2, T = pyr::top_tile(m, pyr::kRestShift);
     int ntx, nty;
     pyr::pass_tiles(g.w, g.h, s, m, T, ntx, nty);
     const int smem = pyr::pass_smem_max(g.w, g.h, s, m, T);
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(pyr_pass_kernel,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > 40 * 1024) {   // 48 KiB less the static part
+      const cudaError_t e = cudaFuncSetAttribute(
+          pyr_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
       if (e != cudaSuccess) return e;
     }
     const long long blocks = (long long)ntx * nty * b.n;
     pyr_pass_kernel<<<(unsigned)blocks, pyr::kThreads, smem, st>>>(g, b, s, m, T, ntx, nty,
                                                                    round_mode);
   }
+  return s + 1 < g.n_levels ? launch_pyramid_from(g, b, s, round_mode, st) : cudaGetLastError();
+}
+
+cudaError_t launch_pyramid_from(const Geom& g, const Batch& b, int s0, int round_mode,
+                                cudaStream_t st, bool* small_out) {
+  bool small = false;   // the previous level's launch left most of the GPU idle
+  for (int s = s0; s + 1 < g.n_levels; ++s) {
+    const int groups = (g.w[s + 1] + 7) / 8, h = g.h[s + 1];
+    // output rows per thread: 8 read 19 input rows for 16 of their own; fewer
+    // while that leaves less than two warps per scheduler
+    int rows = 8;
+    while (rows > 1 && (long long)groups * ((h + rows - 1) / rows) * b.n < 256LL * sm_count())
+      rows >>= 1;
+    const int blocks = (h + rows - 1) / rows;
+    const long long per = (long long)groups * blocks;
+    // 32-bit thread numbers: more images in further launches
+    const int most = (int)std::min<long long>(b.n, std::max<long long>(1, (1LL << 30) / per));
+    for (int i0 = 0; i0 < b.n; i0 += most) {
+      Batch bc = b;
+      bc.l0 += (long long)i0 * b.l0_stride;
+      bc.upper += (long long)i0 * b.upper_stride;
+      bc.n = std::min(most, b.n - i0);
+      const long long threads = per * bc.n;
+      const cudaError_t e = launch_dependent(
+          pyr_level_kernel, dim3((unsigned)((threads + LEVEL_THREADS - 1) / LEVEL_THREADS)),
+          LEVEL_THREADS, 0, st, small && s > s0, g, bc, s, groups, blocks, rows, round_mode);
+      if (e != cudaSuccess) return e;
+      small = threads <= 32LL * kDependentMaxWarpsPerSm * sm_count();
+    }
+  }
+  if (small_out) *small_out = small;
   return cudaGetLastError();
 }
 
-cudaError_t launch_pyramid(const Geom& g, const Batch& b, int round_mode, cudaStream_t s) {
-  return launch_pyramid_from(g, b, 0, round_mode, s);
+cudaError_t launch_pyramid(const Geom& g, const Batch& b, int round_mode, cudaStream_t s,
+                           bool* small) {
+  return launch_pyramid_from(g, b, 0, round_mode, s, small);
 }
 
 }  // namespace vio

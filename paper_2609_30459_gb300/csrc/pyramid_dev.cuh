@@ -361,6 +361,152 @@ __device__ __forceinline__ void pyramid_pass(const Geom& g, const Batch& b, int 
   }
 }
 
+// ---- one level straight from the level below in global memory
+
+// Pixels x .. x + 23 of a row as six words, x + 4 a multiple of 16 (so only the
+// first word can start left of the row), columns outside [0, w) replaced by
+// the edge pixel. `begin`/`end`: the image, for rows at any byte.
+__device__ __forceinline__ void row_words(const uint8_t* __restrict__ row, int x, int w, int al,
+                                          const uint8_t* begin, const uint8_t* end,
+                                          unsigned (&v)[6]) {
+  if ((al & 15) == 0 && x >= 0 && x + 24 <= w) {
+    v[0] = __ldg(reinterpret_cast<const unsigned*>(row + x));
+    const uint4 m = __ldg(reinterpret_cast<const uint4*>(row + x + 4));
+    v[1] = m.x;
+    v[2] = m.y;
+    v[3] = m.z;
+    v[4] = m.w;
+    v[5] = __ldg(reinterpret_cast<const unsigned*>(row + x + 20));
+    return;
+  }
+  if ((al & 3) == 0) {
+    // a word that starts inside the row ends inside its pitch
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int X = x + 4 * k;
+      v[k] = X >= 0 && X < w ? __ldg(reinterpret_cast<const unsigned*>(row + X)) : 0u;
+    }
+  } else {
+    const uint8_t* p = row + x;
+    const unsigned o = (unsigned)(reinterpret_cast<uintptr_t>(p) & 3);
+    unsigned q[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      const uint8_t* a = p - o + 4 * k;
+      q[k] = 0u;
+      if (a >= begin && a + 4 <= end) {
+        q[k] = __ldg(reinterpret_cast<const unsigned*>(a));
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          if (a + b >= begin && a + b < end) q[k] |= (unsigned)__ldg(a + b) << (8 * b);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = __funnelshift_r(q[k], q[k + 1], 8 * o);
+  }
+  if (x < 0) v[0] = (unsigned)__ldg(row) * 0x01010101u;
+  if (x + 24 > w) {
+    const unsigned fill = (unsigned)__ldg(row + w - 1) * 0x01010101u;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int in = w - (x + 4 * k);   // pixels of this word inside the row
+      const unsigned keep = in >= 4 ? 0xffffffffu : (in <= 0 ? 0u : (1u << (8 * in)) - 1u);
+      if (k > 0 || x >= 0) v[k] = (v[k] & keep) | (fill & ~keep);
+    }
+  }
+}
+
+// Eight columns from x0 (a multiple of 8) of output rows y0 .. y0 + n - 1 of
+// level s + 1, from level s: the sums of group8 on registers, each input row
+// unpacked once and added to the two output rows it belongs to.
+__device__ __forceinline__ void level_strip(const Geom& g, const Batch& b, int img, int s, int x0,
+                                            int y0, int n, unsigned add2) {
+  const uint8_t* src = level_ptr(g, b, img, s);
+  const int w = g.w[s], h = g.h[s], pitch = g.pitch[s];
+  uint8_t* dst = level_ptr_mut(g, b, img, s + 1);
+  const int wo = g.w[s + 1], dpitch = g.pitch[s + 1];
+  const bool vec = ((reinterpret_cast<uintptr_t>(dst) | (uintptr_t)dpitch) & 7) == 0;
+  const int al = (int)((reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch) & 15);
+  const uint8_t* end = src + (long long)(h - 1) * pitch + w;
+  auto load = [&](int y, unsigned (&v)[6]) {
+    row_words(src + (long long)clampi(y, 0, h - 1) * pitch, 2 * x0 - 4, w, al, src, end, v);
+  };
+  // sums of output row m (A) and m + 1 (B): even columns [0, 6), odd [6, 11)
+  unsigned A[11], B[11], r[11];
+  auto unpack = [&](const unsigned (&v)[6]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) r[k] = __byte_perm(v[k], 0u, 0x4240);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) r[6 + k] = __byte_perm(v[k], 0u, 0x4341);
+  };
+  unsigned v0[6], v1[6], v2[6];
+  load(2 * y0 - 2, v0);
+  load(2 * y0 - 1, v1);
+  load(2 * y0, v2);
+  unpack(v0);
+#pragma unroll
+  for (int k = 0; k < 11; ++k) A[k] = r[k];
+  unpack(v1);
+#pragma unroll
+  for (int k = 0; k < 11; ++k) A[k] += 4u * r[k];
+  unpack(v2);
+#pragma unroll
+  for (int k = 0; k < 11; ++k) {
+    A[k] += 6u * r[k];
+    B[k] = r[k];
+  }
+  load(2 * y0 + 1, v0);
+  load(2 * y0 + 2, v1);
+#pragma unroll 1
+  for (int m = 0; m < n; ++m) {
+    const int y = y0 + m;
+    unsigned n0[6], n1[6];       // the next output row's two new input rows
+    if (m + 1 < n) {
+      load(2 * y + 3, n0);
+      load(2 * y + 4, n1);
+    }
+    unpack(v0);                  // row 2 y + 1
+#pragma unroll
+    for (int k = 0; k < 11; ++k) {
+      A[k] += 4u * r[k];
+      B[k] += 4u * r[k];
+    }
+    unpack(v1);                  // row 2 y + 2
+#pragma unroll
+    for (int k = 0; k < 11; ++k) A[k] += r[k];
+    unsigned out[4];
+    unsigned L = __byte_perm(A[0], A[1], 0x5432);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned C = __byte_perm(A[i + 1], A[i + 2], 0x5432);
+      const unsigned D = __byte_perm(A[6 + i], A[7 + i], 0x5432);
+      out[i] = L + C + 6u * A[i + 1] + 4u * (D + A[7 + i]) + add2;
+      L = C;
+    }
+    const uint2 q = make_uint2(__byte_perm(out[0], out[1], 0x7531),
+                               __byte_perm(out[2], out[3], 0x7531));
+    uint8_t* d = dst + (long long)y * dpitch + x0;
+    if (vec && x0 + 8 <= wo) {
+      *reinterpret_cast<uint2*>(d) = q;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (x0 + c < wo) d[c] = (uint8_t)((c < 4 ? q.x : q.y) >> (8 * (c & 3)));
+    }
+#pragma unroll
+    for (int k = 0; k < 11; ++k) {
+      A[k] = B[k] + 6u * r[k];
+      B[k] = r[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      v0[k] = n0[k];
+      v1[k] = n1[k];
+    }
+  }
+}
+
 // Tile counts of a pass that ends at level s + m.
 __host__ __device__ inline void pass_tiles(const int* wl, const int* hl, int s, int m, int T,
                                            int& ntx, int& nty) {
@@ -368,9 +514,8 @@ __host__ __device__ inline void pass_tiles(const int* wl, const int* hl, int s, 
   nty = (hl[s + m] + T - 1) / T;
 }
 
-// Passes of the standalone pyramid launches (vio_pyramid_build and the levels
-// a fused launch leaves): two levels each, deepest-level tiles of 32 pixels
-// (a 128 x 128 source region per tile keeps the halo recompute small).
+// Passes of two levels each, deepest-level tiles of 32 pixels (a 128 x 128
+// source region per tile keeps the halo recompute small).
 constexpr int kRestPass = 2;
 constexpr int kRestShift = 1;
 __host__ __device__ inline int rest_pass_levels(int n_levels, int s) {
