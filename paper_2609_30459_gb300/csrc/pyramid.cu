@@ -1,14 +1,15 @@
 // Image pyramid entry point (Sec. III-C, Eq. 1-3): one launch per level, each
 // straight from the level below (level_strip of pyramid_dev.cuh).
 //
-// What bounds it: for a batch larger than the L2, DRAM (level 0 once, the upper
-// levels once; a level's reads find the level before it in the L2); for a few
-// images the launches, which are programmatic dependents of one another. A
-// thread makes eight columns of several rows, so that an input row is loaded
-// and unpacked once or twice and no shared memory or barrier is needed. 185
-// images of 752 x 480 to four levels: PYR_AFTER us; passes of two levels through
-// shared-memory tiles of 128 x 128 pixels took 91 us, bound by the
-// shared-memory wavefronts of every output's 5 x 24 source bytes.
+// What bounds it: the latency of its loads (a thread has all of its rows in
+// flight, 21 loads), for a few images the launches, which are programmatic
+// dependents of one another. A thread makes eight columns of two rows, so that
+// an input row is loaded and unpacked twice and no shared memory or barrier is
+// needed; the inner columns' threads share warps of their own and never test
+// for an edge. 185 images of 752 x 480 to four levels, caches cold: 53 us;
+// passes of two levels through shared-memory tiles of 128 x 128 pixels took 91
+// us, bound by the shared-memory wavefronts of every output's 5 x 24 source
+// bytes.
 #include <algorithm>
 
 #include "pyramid_dev.cuh"
@@ -18,24 +19,35 @@ namespace {
 
 constexpr int LEVEL_THREADS = 128;
 
-// Thread t: strip t of the images' (groups of eight columns) x (blocks of
-// `rows` output rows), columns fastest.
-__global__ void __launch_bounds__(LEVEL_THREADS) pyr_level_kernel(const __grid_constant__ Geom g,
-                                                                  const __grid_constant__ Batch b,
-                                                                  int s, int groups, int blocks,
-                                                                  int rows, int round_mode) {
+// A strip is a group of eight columns x a block of R output rows of an image. Threads first take the inner groups of every image's blocks, columns
+// fastest, then the first and last groups, so that the warps of the former
+// never meet the edge.
+template <int R>
+__global__ void __launch_bounds__(LEVEL_THREADS)
+    pyr_level_kernel(const __grid_constant__ Geom g, const __grid_constant__ Batch b, int s,
+                     int inner, int edge, int blocks, int round_mode) {
   // a programmatic dependent of the level below's launch (no-ops otherwise)
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const unsigned t = blockIdx.x * LEVEL_THREADS + threadIdx.x;
-  const unsigned per = (unsigned)(groups * blocks);
+  const unsigned add2 = round_mode == 0 ? 0x00800080u : 0u;
+  unsigned t = blockIdx.x * LEVEL_THREADS + threadIdx.x;
+  const unsigned n_inner = (unsigned)(inner * blocks) * (unsigned)b.n;
+  const unsigned n_inner_up = (n_inner + 31u) & ~31u;   // edges start a warp of their own
+  const bool at_edge = t >= n_inner_up;
+  if (!at_edge && t >= n_inner) return;
+  if (at_edge) t -= n_inner_up;
+  const unsigned cols = (unsigned)(at_edge ? edge : inner), per = cols * (unsigned)blocks;
   const int img = (int)(t / per);
   if (img >= b.n) return;
-  const int q = (int)(t - (unsigned)img * per);
-  const int by = q / groups, gx = q - by * groups;
-  const int y0 = by * rows;
-  pyr::level_strip(g, b, img, s, 8 * gx, y0, min(rows, g.h[s + 1] - y0),
-                   round_mode == 0 ? 0x00800080u : 0u);
+  const unsigned q = t - (unsigned)img * per;
+  const int by = (int)(q / cols), c = (int)(q - (unsigned)by * cols);
+  const int gx = at_edge ? (c == 0 ? 0 : inner + c) : c + 1;
+  const int y0 = by * R;
+  const uint8_t* src = level_ptr(g, b, img, s);
+  if (!at_edge && ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)g.pitch[s]) & 15) == 0)
+    pyr::level_strip<R, true>(g, b, img, s, 8 * gx, y0, add2);
+  else
+    pyr::level_strip<R, false>(g, b, img, s, 8 * gx, y0, add2);
 }
 
 // Two levels per launch through shared-memory tiles: the deeper levels of a
@@ -77,12 +89,15 @@ cudaError_t launch_pyramid_from(const Geom& g, const Batch& b, int s0, int round
                                 cudaStream_t st, bool* small_out) {
   bool small = false;   // the previous level's launch left most of the GPU idle
   for (int s = s0; s + 1 < g.n_levels; ++s) {
+    // inner groups: the words beside their 16 input columns lie in the level
     const int groups = (g.w[s + 1] + 7) / 8, h = g.h[s + 1];
-    // output rows per thread: 8 read 19 input rows for 16 of their own; fewer
-    // while that leaves less than two warps per scheduler
-    int rows = 8;
-    while (rows > 1 && (long long)groups * ((h + rows - 1) / rows) * b.n < 256LL * sm_count())
-      rows >>= 1;
+    const int inner = std::max(0, std::min(groups - 1, (g.w[s] - 20) / 16 + 1) - 1);
+    const int edge = groups - inner;
+    // output rows per thread: 2 (7 input rows for 4 of their own, all loaded
+    // ahead: 28 us for level 1 of 185 images; 4 rows, 36 us, hold too many
+    // registers to cover the loads), 1 where 2 leave less than two warps per
+    // scheduler
+    const int rows = (long long)groups * ((h + 1) / 2) * b.n < 256LL * sm_count() ? 1 : 2;
     const int blocks = (h + rows - 1) / rows;
     const long long per = (long long)groups * blocks;
     // 32-bit thread numbers: more images in further launches
@@ -92,10 +107,12 @@ cudaError_t launch_pyramid_from(const Geom& g, const Batch& b, int s0, int round
       bc.l0 += (long long)i0 * b.l0_stride;
       bc.upper += (long long)i0 * b.upper_stride;
       bc.n = std::min(most, b.n - i0);
-      const long long threads = per * bc.n;
+      const long long threads = ((long long)inner * blocks * bc.n + 31) / 32 * 32 +
+                                (long long)edge * blocks * bc.n;
       const cudaError_t e = launch_dependent(
-          pyr_level_kernel, dim3((unsigned)((threads + LEVEL_THREADS - 1) / LEVEL_THREADS)),
-          LEVEL_THREADS, 0, st, small && s > s0, g, bc, s, groups, blocks, rows, round_mode);
+          rows == 2 ? pyr_level_kernel<2> : pyr_level_kernel<1>,
+          dim3((unsigned)((threads + LEVEL_THREADS - 1) / LEVEL_THREADS)), LEVEL_THREADS, 0, st,
+          small && s > s0, g, bc, s, inner, edge, blocks, round_mode);
       if (e != cudaSuccess) return e;
       small = threads <= 32LL * kDependentMaxWarpsPerSm * sm_count();
     }

@@ -365,20 +365,11 @@ __device__ __forceinline__ void pyramid_pass(const Geom& g, const Batch& b, int 
 
 // Pixels x .. x + 23 of a row as six words, x + 4 a multiple of 16 (so only the
 // first word can start left of the row), columns outside [0, w) replaced by
-// the edge pixel. `begin`/`end`: the image, for rows at any byte.
+// the edge pixel. al: the row addresses' low four bits or'ed. `begin`/`end`:
+// the image, for rows at any byte.
 __device__ __forceinline__ void row_words(const uint8_t* __restrict__ row, int x, int w, int al,
                                           const uint8_t* begin, const uint8_t* end,
                                           unsigned (&v)[6]) {
-  if ((al & 15) == 0 && x >= 0 && x + 24 <= w) {
-    v[0] = __ldg(reinterpret_cast<const unsigned*>(row + x));
-    const uint4 m = __ldg(reinterpret_cast<const uint4*>(row + x + 4));
-    v[1] = m.x;
-    v[2] = m.y;
-    v[3] = m.z;
-    v[4] = m.w;
-    v[5] = __ldg(reinterpret_cast<const unsigned*>(row + x + 20));
-    return;
-  }
   if ((al & 3) == 0) {
     // a word that starts inside the row ends inside its pitch
 #pragma unroll
@@ -417,92 +408,85 @@ __device__ __forceinline__ void row_words(const uint8_t* __restrict__ row, int x
   }
 }
 
-// Eight columns from x0 (a multiple of 8) of output rows y0 .. y0 + n - 1 of
-// level s + 1, from level s: the sums of group8 on registers, each input row
-// unpacked once and added to the two output rows it belongs to.
+// Eight columns from x0 (a multiple of 8) of output rows y0 .. y0 + R - 1 (those
+// inside the level) of level s + 1, from level s: the sums of group8 on
+// registers, each input row unpacked once and added to the two output rows it
+// belongs to; all 2 R + 3 rows are loaded before the first is used. INNER:
+// every input column and the two words beside them lie inside the level and
+// its rows start on 16-byte boundaries.
+template <int R, bool INNER>
 __device__ __forceinline__ void level_strip(const Geom& g, const Batch& b, int img, int s, int x0,
-                                            int y0, int n, unsigned add2) {
+                                            int y0, unsigned add2) {
   const uint8_t* src = level_ptr(g, b, img, s);
   const int w = g.w[s], h = g.h[s], pitch = g.pitch[s];
   uint8_t* dst = level_ptr_mut(g, b, img, s + 1);
-  const int wo = g.w[s + 1], dpitch = g.pitch[s + 1];
+  const int wo = g.w[s + 1], ho = g.h[s + 1], dpitch = g.pitch[s + 1];
   const bool vec = ((reinterpret_cast<uintptr_t>(dst) | (uintptr_t)dpitch) & 7) == 0;
-  const int al = (int)((reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch) & 15);
-  const uint8_t* end = src + (long long)(h - 1) * pitch + w;
-  auto load = [&](int y, unsigned (&v)[6]) {
-    row_words(src + (long long)clampi(y, 0, h - 1) * pitch, 2 * x0 - 4, w, al, src, end, v);
-  };
+  unsigned v[2 * R + 3][6];
+  if (INNER) {
+#pragma unroll
+    for (int i = 0; i < 2 * R + 3; ++i) {
+      const uint8_t* p = src + (long long)clampi(2 * y0 - 2 + i, 0, h - 1) * pitch + 2 * x0;
+      v[i][0] = __ldg(reinterpret_cast<const unsigned*>(p - 4));
+      const uint4 m = __ldg(reinterpret_cast<const uint4*>(p));
+      v[i][1] = m.x;
+      v[i][2] = m.y;
+      v[i][3] = m.z;
+      v[i][4] = m.w;
+      v[i][5] = __ldg(reinterpret_cast<const unsigned*>(p + 16));
+    }
+  } else {
+    const int al = (int)((reinterpret_cast<uintptr_t>(src) | (uintptr_t)pitch) & 15);
+    const uint8_t* end = src + (long long)(h - 1) * pitch + w;
+#pragma unroll
+    for (int i = 0; i < 2 * R + 3; ++i)
+      row_words(src + (long long)clampi(2 * y0 - 2 + i, 0, h - 1) * pitch, 2 * x0 - 4, w, al, src,
+                end, v[i]);
+  }
   // sums of output row m (A) and m + 1 (B): even columns [0, 6), odd [6, 11)
-  unsigned A[11], B[11], r[11];
-  auto unpack = [&](const unsigned (&v)[6]) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) r[k] = __byte_perm(v[k], 0u, 0x4240);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) r[6 + k] = __byte_perm(v[k], 0u, 0x4341);
+  unsigned A[11], B[11];
+  auto lane2 = [&](int i, int k) {   // 16-bit lanes k of input row i
+    return k < 6 ? __byte_perm(v[i][k], 0u, 0x4240) : __byte_perm(v[i][k - 6], 0u, 0x4341);
   };
-  unsigned v0[6], v1[6], v2[6];
-  load(2 * y0 - 2, v0);
-  load(2 * y0 - 1, v1);
-  load(2 * y0, v2);
-  unpack(v0);
-#pragma unroll
-  for (int k = 0; k < 11; ++k) A[k] = r[k];
-  unpack(v1);
-#pragma unroll
-  for (int k = 0; k < 11; ++k) A[k] += 4u * r[k];
-  unpack(v2);
 #pragma unroll
   for (int k = 0; k < 11; ++k) {
-    A[k] += 6u * r[k];
-    B[k] = r[k];
+    const unsigned c = lane2(2, k);
+    A[k] = lane2(0, k) + 4u * lane2(1, k) + 6u * c;
+    B[k] = c;
   }
-  load(2 * y0 + 1, v0);
-  load(2 * y0 + 2, v1);
-#pragma unroll 1
-  for (int m = 0; m < n; ++m) {
+#pragma unroll
+  for (int m = 0; m < R; ++m) {
     const int y = y0 + m;
-    unsigned n0[6], n1[6];       // the next output row's two new input rows
-    if (m + 1 < n) {
-      load(2 * y + 3, n0);
-      load(2 * y + 4, n1);
-    }
-    unpack(v0);                  // row 2 y + 1
 #pragma unroll
     for (int k = 0; k < 11; ++k) {
-      A[k] += 4u * r[k];
-      B[k] += 4u * r[k];
+      const unsigned o = lane2(2 * m + 3, k), c = lane2(2 * m + 4, k);
+      const unsigned t = A[k] + 4u * o + c;
+      A[k] = B[k] + 4u * o + 6u * c;   // the next output row's, so far
+      B[k] = c;
+      if (k < 6) v[0][k] = t; else v[1][k - 6] = t;   // rows 0 and 1 hold the sums now
     }
-    unpack(v1);                  // row 2 y + 2
-#pragma unroll
-    for (int k = 0; k < 11; ++k) A[k] += r[k];
+    const unsigned* E = v[0];
+    const unsigned* O = v[1];
     unsigned out[4];
-    unsigned L = __byte_perm(A[0], A[1], 0x5432);
+    unsigned L = __byte_perm(E[0], E[1], 0x5432);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const unsigned C = __byte_perm(A[i + 1], A[i + 2], 0x5432);
-      const unsigned D = __byte_perm(A[6 + i], A[7 + i], 0x5432);
-      out[i] = L + C + 6u * A[i + 1] + 4u * (D + A[7 + i]) + add2;
+      const unsigned C = __byte_perm(E[i + 1], E[i + 2], 0x5432);
+      const unsigned D = __byte_perm(O[i], O[i + 1], 0x5432);
+      out[i] = L + C + 6u * E[i + 1] + 4u * (D + O[i + 1]) + add2;
       L = C;
     }
     const uint2 q = make_uint2(__byte_perm(out[0], out[1], 0x7531),
                                __byte_perm(out[2], out[3], 0x7531));
-    uint8_t* d = dst + (long long)y * dpitch + x0;
-    if (vec && x0 + 8 <= wo) {
-      *reinterpret_cast<uint2*>(d) = q;
-    } else {
+    if (y < ho) {
+      uint8_t* d = dst + (long long)y * dpitch + x0;
+      if (vec && x0 + 8 <= wo) {
+        *reinterpret_cast<uint2*>(d) = q;
+      } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (x0 + c < wo) d[c] = (uint8_t)((c < 4 ? q.x : q.y) >> (8 * (c & 3)));
-    }
-#pragma unroll
-    for (int k = 0; k < 11; ++k) {
-      A[k] = B[k] + 6u * r[k];
-      B[k] = r[k];
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      v0[k] = n0[k];
-      v1[k] = n1[k];
+        for (int c = 0; c < 8; ++c)
+          if (x0 + c < wo) d[c] = (uint8_t)((c < 4 ? q.x : q.y) >> (8 * (c & 3)));
+      }
     }
   }
 }
