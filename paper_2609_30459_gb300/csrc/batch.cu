@@ -494,8 +494,12 @@ extern "C" vio_status vio_batch_get_view(vio_batch* b, int32_t g, vio_frontend_v
 extern "C" int32_t vio_batch_launches_per_step(const vio_batch* b) {
   if (!b) return 0;
   std::vector<vio::Geom> g;
-  for (const auto& G : b->groups) g.push_back(vio::make_geom(G.layout));
-  return vio::frame_launches(g.data(), (int)g.size(), b->net != nullptr,
+  std::vector<int> ns;
+  for (const auto& G : b->groups) {
+    g.push_back(vio::make_geom(G.layout));
+    ns.push_back(G.spec.n_streams);
+  }
+  return vio::frame_launches(g.data(), ns.data(), (int)g.size(), b->net != nullptr,
                             b->tune.stereo_after != 0, b->tune.pyr_first);
 }
 

@@ -109,7 +109,10 @@ __global__ void __launch_bounds__(NT, 768 / NT) frame_front_kernel(const __grid_
   const int rem = (int)(b - (long long)unit * a.blocks_per_unit);
   int base = unit * a.det_step;
   if (a.det_step == 2 && a.slotted) {
-    if (a.active && a.active[unit] == 0) return;
+    if (a.active && a.active[unit] == 0) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      return;
+    }
     base = 2 * (a.parity[unit] * a.n_streams + unit);
   }
   const int tiles = a.ntx * a.nty;
@@ -127,6 +130,44 @@ __global__ void __launch_bounds__(NT, 768 / NT) frame_front_kernel(const __grid_
                             MASKED ? a.mask + (long long)unit * a.mask_stride : nullptr,
                             a.cand + (long long)unit * a.n_cells * a.cg.k,
                             a.cand_count + (long long)unit * a.n_cells, smem);
+  // after the level launches of a split front (a no-op otherwise): they read
+  // the same frames and write nothing this launch reads, so it ran beside them
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// One pyramid level of both cameras of every active stream of every group (the
+// front of a large step, see split_front): level s + 1 from level s, two
+// output rows per thread (level_strip of pyramid_dev.cuh).
+struct LevelGroup {
+  Geom g;
+  Batch all;
+  int slotted, n_streams, round_mode;
+  const int32_t* parity;
+  const int32_t* active;
+  pyr::Strips p;
+};
+struct MultiLevel {
+  int n, s;
+  long long block_end[kMaxGroups];
+  LevelGroup a[kMaxGroups];
+};
+constexpr int LEVEL_THREADS = 128;
+__global__ void __launch_bounds__(LEVEL_THREADS)
+    frame_level_kernel(const __grid_constant__ MultiLevel mm) {
+  // a programmatic dependent of the level below's launch (no-ops otherwise)
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  long long start;
+  const int gi = group_of(mm, blockIdx.x, start);
+  const LevelGroup& a = mm.a[gi];
+  pyr::make_strip<2>(a.g, a.all, mm.s, a.p,
+                     (unsigned)(blockIdx.x - start) * LEVEL_THREADS + threadIdx.x,
+                     2 * a.n_streams, a.round_mode, [&](int i) {
+                       const int unit = i >> 1;
+                       if (!a.slotted) return i;
+                       if (a.active && a.active[unit] == 0) return -1;
+                       return 2 * (a.parity[unit] * a.n_streams + unit) + (i & 1);
+                     });
 }
 
 struct MultiK2 {
@@ -504,8 +545,25 @@ __global__ void __launch_bounds__(K3_THREADS)
   }
 }
 
-// Levels the fused pass of K1 computes (the rest follow in further passes).
+// The front of a large step: a launch per pyramid level and then the detection
+// alone, in place of one launch of tiles that compute up to four levels each
+// beside the detection blocks. The fused launch saves launches where they
+// are the time (one 752 x 480 frame: 15 us against 28 us in four launches),
+// but recomputes halos and runs both parts at the larger one's shared memory
+// and registers: the 16 mixed streams of a batch (29 million pixels) took 301
+// us fused, 97 us split; two 1920 x 1080 pairs (8 million) 75 and 58 us. Only
+// when the levels of the fused pass are left to this rule (pyr_first 0).
+constexpr long long kSplitPixels = 4LL << 20;
+bool split_front(const Geom* g, const int* n_streams, int n_groups, int pyr_first) {
+  long long px = 0;
+  for (int i = 0; i < n_groups; ++i) px += 2LL * n_streams[i] * g[i].w[0] * g[i].h[0];
+  return pyr_first == 0 && px >= kSplitPixels;
+}
+
+// Levels the fused pass of K1 computes (the rest follow in further passes);
+// pyr_first < 0: none.
 int first_levels(const Geom& g, int pyr_first) {
+  if (pyr_first < 0) return 0;
   const int m = g.n_levels > 1 ? pyr::pass_levels(g.n_levels, 0) : 0;
   return (pyr_first > 0 && pyr_first < m) ? pyr_first : m;
 }
@@ -539,26 +597,28 @@ K1Args front_args(const vio_params& p, const Geom& g, const Batch& all, int det_
 }
 
 template <int NT, bool MASKED>
-cudaError_t launch_k1_nt(const MultiK1& mm, int smem, cudaStream_t s) {
+cudaError_t launch_k1_nt(const MultiK1& mm, int smem, cudaStream_t s, bool beside) {
   if (smem > 40 * 1024) {   // 48 KiB less the static part
     const cudaError_t e = cudaFuncSetAttribute(
         frame_front_kernel<NT, MASKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
   const long long blocks = mm.block_end[mm.n - 1];
-  if (blocks > 0) frame_front_kernel<NT, MASKED><<<(unsigned)blocks, NT, smem, s>>>(mm);
-  return cudaGetLastError();
+  if (blocks <= 0) return cudaSuccess;
+  return launch_dependent(frame_front_kernel<NT, MASKED>, dim3((unsigned)blocks), NT, (size_t)smem,
+                          s, beside, mm);
 }
 
-// MASKED when any group of the launch has a per-pixel detection mask.
-cudaError_t launch_k1(const MultiK1& mm, int smem, int threads, cudaStream_t s) {
+// MASKED when any group of the launch has a per-pixel detection mask. beside:
+// as a programmatic dependent of the level launches.
+cudaError_t launch_k1(const MultiK1& mm, int smem, int threads, cudaStream_t s, bool beside) {
   bool masked = false;
   for (int i = 0; i < mm.n; ++i) masked = masked || mm.a[i].mask != nullptr;
   if (masked)
-    return threads == 128 ? launch_k1_nt<128, true>(mm, smem, s)
-                          : launch_k1_nt<256, true>(mm, smem, s);
-  return threads == 128 ? launch_k1_nt<128, false>(mm, smem, s)
-                        : launch_k1_nt<256, false>(mm, smem, s);
+    return threads == 128 ? launch_k1_nt<128, true>(mm, smem, s, beside)
+                          : launch_k1_nt<256, true>(mm, smem, s, beside);
+  return threads == 128 ? launch_k1_nt<128, false>(mm, smem, s, beside)
+                        : launch_k1_nt<256, false>(mm, smem, s, beside);
 }
 
 }  // namespace
@@ -587,6 +647,15 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
   if (part != 2) {
     // K1: pyramid levels 1-4 + detection candidates (camera 0 of each stream)
     mark(0);
+    Geom geoms[kMaxGroups];
+    int ns[kMaxGroups];
+    for (int i = 0; i < n_groups; ++i) {
+      geoms[i] = fl[i].g;
+      ns[i] = fl[i].n_streams;
+    }
+    const bool split = split_front(geoms, ns, n_groups, tune.pyr_first);
+    const int pyr_first = split ? -1 : tune.pyr_first;
+    const int k1_threads = split ? 128 : tune.k1_threads;
     MultiK1 m1{};
     m1.n = n_groups;
     int smem1 = 0;
@@ -598,7 +667,7 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     for (int i = 0; i < n_groups; ++i) {
       const FrameLaunch& f = fl[i];
       K1Args a = front_args(f.p, f.g, f.cur, 2, nullptr, 0, f.cand, f.cand_count,
-                            tune.pyr_tile_shift, tune.pyr_first, tune.k1_threads, gw);
+                            tune.pyr_tile_shift, pyr_first, k1_threads, gw);
       a.slotted = f.slotted;
       a.n_streams = f.n_streams;
       a.parity = f.parity;
@@ -608,15 +677,38 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
       m1.a[i] = a;
       acc += (long long)f.n_streams * a.blocks_per_unit;
       m1.block_end[i] = acc;
-      const int sm = frame_front_smem(f.g, f.p, tune.pyr_tile_shift, tune.pyr_first,
-                                      tune.k1_threads, gw);
+      const int sm = frame_front_smem(f.g, f.p, tune.pyr_tile_shift, pyr_first, k1_threads, gw);
       smem1 = sm > smem1 ? sm : smem1;
     }
-    e = launch_k1(m1, smem1, tune.k1_threads, s);
+    // beside one another as programmatic dependents, while the detection is
+    // about one wave of CTAs (two 1920 x 1080 pairs, pipelined over four frames:
+    // 734 to 715 us; the batch's 2240 CTAs: 675 us so, 699 us beside)
+    const bool beside = split && acc <= 8LL * sm_count();
+    for (int lv = 0; split; ++lv) {
+      MultiLevel ml{};
+      ml.n = n_groups;
+      ml.s = lv;
+      acc = 0;
+      for (int i = 0; i < n_groups; ++i) {
+        const FrameLaunch& f = fl[i];
+        if (lv + 1 < f.g.n_levels) {
+          ml.a[i] = LevelGroup{f.g, f.cur, f.slotted, f.n_streams, f.p.round_mode, f.parity,
+                               f.active, pyr::strips(f.g, lv, 2)};
+          acc += (pyr::strip_threads(ml.a[i].p, 2 * f.n_streams) + LEVEL_THREADS - 1) /
+                 LEVEL_THREADS;
+        }
+        ml.block_end[i] = acc;
+      }
+      if (acc == 0) break;
+      e = launch_dependent(frame_level_kernel, dim3((unsigned)acc), LEVEL_THREADS, 0, s,
+                           beside && lv > 0, ml);
+      if (e != cudaSuccess) return e;
+    }
+    e = launch_k1(m1, smem1, k1_threads, s, beside);
     if (e != cudaSuccess) return e;
     // levels beyond the first pass
     mark(1);
-    for (int i = 0; i < n_groups; ++i) {
+    for (int i = 0; i < n_groups && !split; ++i) {
       const FrameLaunch& f = fl[i];
       const int m1 = first_levels(f.g, tune.pyr_first);
       if (f.g.n_levels > 1 + m1) {
@@ -727,9 +819,14 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
   return cudaGetLastError();
 }
 
-int frame_launches(const Geom* g, int n_groups, bool with_net, bool stereo_after,
-                   int pyr_first) {
+int frame_launches(const Geom* g, const int* n_streams, int n_groups, bool with_net,
+                   bool stereo_after, int pyr_first) {
   int n = (with_net ? 4 : 3) + (stereo_after ? 2 : 0);   // K1, (KN), K2, K3, (K4, K5)
+  if (split_front(g, n_streams, n_groups, pyr_first)) {
+    int levels = 0;
+    for (int i = 0; i < n_groups; ++i) levels = levels > g[i].n_levels ? levels : g[i].n_levels;
+    return n + levels - 1;
+  }
   for (int i = 0; i < n_groups; ++i) {
     const int rest = g[i].n_levels - 1 - first_levels(g[i], pyr_first);
     if (rest > 0) n += pyr::rest_passes(rest);

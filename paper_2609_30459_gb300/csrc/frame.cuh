@@ -96,7 +96,7 @@ __host__ __device__ inline StreamRef stream_ref(const FrameLaunch& f, int s) {
 
 // Enqueues one frame of every group on `s` (3 launches, plus one pyramid
 // pass per group for levels beyond 5, plus the flow proposals when the
-// groups' initializer is on). marks: VIO_N_STAGES + 1 events recorded at the
+// groups' initializer is on; large steps have a launch per pyramid level). marks: VIO_N_STAGES + 1 events recorded at the
 // stage boundaries (or null).
 // part: 0 the whole step; 1 only its front (pyramids and detection
 // candidates: K1 and the deeper pyramid levels); 2 the rest. The front of a
@@ -105,8 +105,8 @@ __host__ __device__ inline StreamRef stream_ref(const FrameLaunch& f, int s) {
 // when those are not the previous step's.
 cudaError_t launch_frames(const FrameLaunch* f, int n_groups, const FrameTune& tune,
                           cudaStream_t s, cudaEvent_t* marks, int part = 0);
-int frame_launches(const Geom* g, int n_groups, bool with_net, bool stereo_after,
-                   int pyr_first);
+int frame_launches(const Geom* g, const int* n_streams, int n_groups, bool with_net,
+                   bool stereo_after, int pyr_first);
 
 // Keypoint lists (2 per stream) one launch of the proposal kernel handles.
 constexpr int KN_MAX_LISTS = 256;

@@ -250,7 +250,8 @@ extern "C" int32_t vio_frontend_launches_per_step(const vio_frontend* fe) {
   vio_pyr_layout L;
   if (vio_pyr_layout_make(fe->w, fe->h, fe->p.n_levels, fe->w, &L) != VIO_OK) return 0;
   const vio::Geom g = vio::make_geom(L);
-  return vio::frame_launches(&g, 1, fe->net != nullptr, false, fe->tune.pyr_first);
+  return vio::frame_launches(&g, &fe->n_streams, 1, fe->net != nullptr, false,
+                            fe->tune.pyr_first);
 }
 
 extern "C" vio_status vio_frontend_set_tune(vio_frontend* fe, const vio_batch_tune* t) {

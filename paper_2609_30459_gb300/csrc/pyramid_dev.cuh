@@ -491,6 +491,52 @@ __device__ __forceinline__ void level_strip(const Geom& g, const Batch& b, int i
   }
 }
 
+// Numbering of a level launch's strips (a group of eight columns x a block of R
+// output rows of an image): first the inner groups of every image's blocks,
+// columns fastest, then, from the next warp on, the first and last groups, so
+// that the warps of the former never meet the edge.
+struct Strips {
+  int inner, edge, blocks;   // groups per row, blocks of rows
+};
+inline Strips strips(const Geom& g, int s, int rows) {
+  // inner groups: the words beside their 16 input columns lie in the level
+  const int groups = (g.w[s + 1] + 7) / 8;
+  Strips p;
+  p.inner = std::max(0, std::min(groups - 1, (g.w[s] - 20) / 16 + 1) - 1);
+  p.edge = groups - p.inner;
+  p.blocks = (g.h[s + 1] + rows - 1) / rows;
+  return p;
+}
+inline long long strip_threads(const Strips& p, int n_images) {
+  return ((long long)p.inner * p.blocks * n_images + 31) / 32 * 32 +
+         (long long)p.edge * p.blocks * n_images;
+}
+// Makes strip t of a launch over n images of level s + 1; f(i) is the batch index
+// of the launch's image i, negative to leave it out.
+template <int R, class F>
+__device__ __forceinline__ void make_strip(const Geom& g, const Batch& b, int s, const Strips& p,
+                                           unsigned t, int n, int round_mode, F f) {
+  const unsigned n_inner = (unsigned)(p.inner * p.blocks) * (unsigned)n;
+  const unsigned n_inner_up = (n_inner + 31u) & ~31u;
+  const bool at_edge = t >= n_inner_up;
+  if (!at_edge && t >= n_inner) return;
+  if (at_edge) t -= n_inner_up;
+  const unsigned cols = (unsigned)(at_edge ? p.edge : p.inner), per = cols * (unsigned)p.blocks;
+  const int i = (int)(t / per);
+  if (i >= n) return;
+  const unsigned q = t - (unsigned)i * per;
+  const int by = (int)(q / cols), c = (int)(q - (unsigned)by * cols);
+  const int gx = at_edge ? (c == 0 ? 0 : p.inner + c) : c + 1;
+  const int img = f(i);
+  if (img < 0) return;
+  const unsigned add2 = round_mode == 0 ? 0x00800080u : 0u;
+  const uint8_t* src = level_ptr(g, b, img, s);
+  if (!at_edge && ((reinterpret_cast<uintptr_t>(src) | (uintptr_t)g.pitch[s]) & 15) == 0)
+    level_strip<R, true>(g, b, img, s, 8 * gx, by * R, add2);
+  else
+    level_strip<R, false>(g, b, img, s, 8 * gx, by * R, add2);
+}
+
 // Tile counts of a pass that ends at level s + m.
 __host__ __device__ inline void pass_tiles(const int* wl, const int* hl, int s, int m, int T,
                                            int& ntx, int& nty) {
