@@ -46,7 +46,7 @@
 #include "initnet_dev.cuh"
 #include "initnet_tc.cuh"
 #include "pyramid_dev.cuh"
-#include "track_dev.cuh"
+#include "track_group.cuh"
 
 namespace vio {
 namespace {
@@ -421,6 +421,126 @@ __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ Mult
   }
 }
 
+// The items of frame_track_kernel (temporal tracks and stereo candidates of
+// every group, in its numbering) for the grouped tracker.
+struct FrameTracks {
+  const MultiK2& mm;
+  struct Ref {
+    long long out;        // temporal or stereo slot of the group
+    int gi, s_img, d_img; // group, source and target image
+    bool temporal, learned;
+  };
+  __device__ __forceinline__ long long total() const { return mm.block_end[mm.n - 1]; }
+  __device__ __forceinline__ bool fetch(long long w, bool lead, Ref& ref, trk::Task& K) const {
+    long long start;
+    ref.gi = group_of(mm, w, start);
+    const FrameLaunch& f = mm.f[ref.gi];
+    const long long wl = w - start;
+    const long long n_temporal = 2LL * f.n_streams * f.cap;
+    ref.temporal = wl < n_temporal;
+    ref.learned = false;
+    K.has_init = false;
+    K.top = f.g.n_levels - 1;
+    K.iters = f.p.gn_iters;
+    K.fb = 1;
+    K.fb_max = f.p.fb_max_dist;
+    if (ref.temporal) {
+      const int list = (int)(wl / f.cap);       // 2s + c
+      const int slot = (int)(wl - (long long)list * f.cap);
+      const int s = list >> 1, c = list & 1;
+      const StreamRef r = stream_ref(f, s);
+      if (!r.active) return false;
+      ref.out = wl;
+      const long long in_list = ((long long)r.li * f.n_streams + s) * 2 + c;
+      if (!r.have_prev || slot >= f.list_count[in_list]) {
+        if (lead) f.trk_status[wl] = VIO_TRACK_EMPTY;
+        return false;
+      }
+      const long long src = in_list * f.cap + slot;
+      K.px = f.list_xy[2 * src];
+      K.py = f.list_xy[2 * src + 1];
+      ref.s_img = r.prev_img + c;
+      ref.d_img = r.cur_img + c;
+      if (f.net) {
+        const float* q = f.net_out + 3 * wl;
+        if (q[2] >= f.net_tau) {
+          ref.learned = true;
+          K.has_init = true;
+          K.ix = K.px + q[0];
+          K.iy = K.py + q[1];
+          K.ith = 0.f;
+          K.top = f.net_top;
+        }
+      }
+      return true;
+    }
+    const long long w2 = wl - n_temporal;
+    const int k = f.p.k_per_cell;
+    const int n_cells = (f.g.w[0] / f.p.cell_w) * (f.g.h[0] / f.p.cell_h);
+    const int per = n_cells * k;
+    const int s = (int)(w2 / per);
+    const int rem = (int)(w2 - (long long)s * per);
+    const int cell = rem / k, rr = rem - cell * k;
+    const StreamRef r = stream_ref(f, s);
+    if (!r.active) return false;
+    ref.out = w2;
+    if (rr >= f.cand_count[(long long)s * n_cells + cell]) {
+      if (lead) f.spec_status[w2] = VIO_TRACK_EMPTY;
+      return false;
+    }
+    const unsigned idx = ~(unsigned)(f.cand[w2] & 0xffffffffu);
+    K.px = (float)(idx % (unsigned)f.g.w[0]);
+    K.py = (float)(idx / (unsigned)f.g.w[0]);
+    ref.s_img = r.cur_img;
+    ref.d_img = r.cur_img + 1;
+    return true;
+  }
+  __device__ __forceinline__ void levels(const Ref& ref, bool back, int l, trk::Lv& S,
+                                         trk::Lv& D) const {
+    const FrameLaunch& f = mm.f[ref.gi];
+    const Batch& from = ref.temporal ? f.prev : f.cur;
+    S = trk::get_lv(f.g, back ? f.cur : from, back ? ref.d_img : ref.s_img, l);
+    D = trk::get_lv(f.g, back ? from : f.cur, back ? ref.s_img : ref.d_img, l);
+  }
+  __device__ __forceinline__ bool finish(Ref& ref, bool lead, const trk::TrackResult& R,
+                                         trk::Task& K) const {
+    const FrameLaunch& f = mm.f[ref.gi];
+    bool learned = ref.learned;
+    if (learned) {
+      learned = R.status == VIO_TRACK_OK && !(f.net_max_step > 0.f && R.last > f.net_max_step);
+      if (!learned) {   // the plain track
+        ref.learned = false;
+        K.has_init = false;
+        K.top = f.g.n_levels - 1;
+        return false;
+      }
+    }
+    if (lead) {
+      if (ref.temporal) {
+        if (f.net) f.trk_learned[ref.out] = learned ? 1 : 0;
+        f.trk_status[ref.out] = (uint8_t)R.status;
+        f.trk_xy[2 * ref.out] = R.x;
+        f.trk_xy[2 * ref.out + 1] = R.y;
+      } else {
+        f.spec_status[ref.out] = (uint8_t)R.status;
+        f.spec_xy[2 * ref.out] = R.x;
+        f.spec_xy[2 * ref.out + 1] = R.y;
+      }
+    }
+    return true;
+  }
+};
+
+__global__ void __launch_bounds__(trk::kGroupThreads, trk::kGroupCtasPerSm)
+    frame_track_groups_kernel(const __grid_constant__ MultiK2 mm) {
+  constexpr int WPB = trk::kGroupThreads / 32;
+  __shared__ __align__(16) uint8_t smem[WPB * trk::kWarpBytes<trk::kGroupLanes>];
+  const int warp = threadIdx.x >> 5;
+  trk::run_tracks<trk::kGroupLanes>(FrameTracks{mm}, (long long)blockIdx.x * WPB + warp,
+                                    (long long)gridDim.x * WPB,
+                                    smem + warp * trk::kWarpBytes<trk::kGroupLanes>);
+}
+
 struct MultiK3 {
   int n;
   long long block_end[kMaxGroups];   // in blocks (= streams)
@@ -560,6 +680,11 @@ bool split_front(const Geom* g, const int* n_streams, int n_groups, int pyr_firs
   return pyr_first == 0 && px >= kSplitPixels;
 }
 
+// Slots of a step's tracking launch per SM from which it runs by groups of lanes
+// (track_group.cuh) instead of a warp per keypoint: 28 keypoints, and about
+// three in five slots of a step hold one.
+constexpr long long kGroupSlotsPerSm = 46;
+
 // Levels the fused pass of K1 computes (the rest follow in further passes);
 // pyr_first < 0: none.
 int first_levels(const Geom& g, int pyr_first) {
@@ -683,7 +808,7 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     // beside one another as programmatic dependents, while the detection is
     // about one wave of CTAs (two 1920 x 1080 pairs, pipelined over four frames:
     // 734 to 715 us; the batch's 2240 CTAs: 675 us so, 699 us beside)
-    const bool beside = split && acc <= 8LL * sm_count();
+    bool beside = split && acc <= 8LL * sm_count();
     for (int lv = 0; split; ++lv) {
       MultiLevel ml{};
       ml.n = n_groups;
@@ -699,7 +824,10 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
         }
         ml.block_end[i] = acc;
       }
-      if (acc == 0) break;
+      if (acc == 0) {
+        beside = beside && lv > 0;
+        break;
+      }
       e = launch_dependent(frame_level_kernel, dim3((unsigned)acc), LEVEL_THREADS, 0, s,
                            beside && lv > 0, ml);
       if (e != cudaSuccess) return e;
@@ -764,7 +892,9 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
   const bool k2_small = acc <= (long long)kDependentMaxWarpsPerSm * sm_count();
   if (acc > 0) {
     const long long blocks2 = (acc * 32 + k2t - 1) / k2t;
-    if (k2_small)
+    if (acc >= kGroupSlotsPerSm * sm_count())
+      frame_track_groups_kernel<<<(unsigned)trk::group_ctas(acc), trk::kGroupThreads, 0, s>>>(m2);
+    else if (k2_small)
       frame_track_kernel<true><<<(unsigned)blocks2, k2t, 0, s>>>(m2);
     else
       frame_track_kernel<false><<<(unsigned)blocks2, k2t, 0, s>>>(m2);

@@ -1,7 +1,8 @@
 // Pyramidal inverse-compositional KLT (Sec. III-E, Eq. 4-5) for the stage
 // entry points vio_track_patches / vio_stereo_match, and the
-// forward-backward distance check. The tracker itself is in track_dev.cuh.
-#include "track_dev.cuh"
+// forward-backward distance check. The tracker itself is in track_dev.cuh (a
+// warp per keypoint) and track_group.cuh (large launches).
+#include "track_group.cuh"
 
 namespace vio {
 namespace {
@@ -24,7 +25,7 @@ struct TrackArgs {
 
 constexpr int TRK_THREADS = 128;
 
-__global__ void __launch_bounds__(TRK_THREADS) track_kernel(TrackArgs a) {
+__global__ void __launch_bounds__(TRK_THREADS) track_kernel(const __grid_constant__ TrackArgs a) {
   const long long wid = ((long long)blockIdx.x * TRK_THREADS + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   const long long total = (long long)a.capacity * a.n_images;
@@ -70,6 +71,79 @@ __global__ void __launch_bounds__(TRK_THREADS) track_kernel(TrackArgs a) {
   }
 }
 
+// Keypoint wid = image * capacity + slot.
+struct StageSource {
+  const TrackArgs& a;
+  struct Ref {
+    long long wid;
+    int img;
+  };
+  __device__ __forceinline__ long long total() const {
+    return (long long)a.capacity * a.n_images;
+  }
+  __device__ __forceinline__ bool fetch(long long wid, bool lead, Ref& ref, trk::Task& K) const {
+    const int img = (int)(wid / a.capacity);
+    const int k = (int)(wid - (long long)img * a.capacity);
+    const int n = a.count ? min(a.count[a.shared_pts ? 0 : img], a.capacity) : a.capacity;
+    ref.wid = wid;
+    ref.img = img;
+    if (k >= n) {
+      const float nanf_ = __int_as_float(0x7fc00000);
+      if (lead) write(wid, trk::TrackResult{VIO_TRACK_EMPTY, false, nanf_, nanf_, nanf_, nanf_,
+                                            nanf_});
+      return false;
+    }
+    const long long pk = a.shared_pts ? k : wid;   // keypoint slot of the source list
+    K.px = a.pts[2 * pk];
+    K.py = a.pts[2 * pk + 1];
+    K.has_init = a.init != nullptr;
+    if (K.has_init) {
+      K.ix = a.init[3 * wid];
+      K.iy = a.init[3 * wid + 1];
+      K.ith = a.init[3 * wid + 2];
+    }
+    K.top = top_level(a.cfg, a.g);
+    K.iters = a.cfg.gn_iters;
+    K.fb = a.cfg.fb;
+    K.fb_max = a.cfg.fb_max_dist;
+    return true;
+  }
+  __device__ __forceinline__ void levels(const Ref& ref, bool back, int l, trk::Lv& S,
+                                         trk::Lv& D) const {
+    S = trk::get_lv(a.g, back ? a.dst : a.src, ref.img, l);
+    D = trk::get_lv(a.g, back ? a.src : a.dst, ref.img, l);
+  }
+  __device__ __forceinline__ bool finish(const Ref& ref, bool lead, const trk::TrackResult& R,
+                                         trk::Task&) const {
+    if (lead) write(ref.wid, R);
+    return true;
+  }
+  __device__ __forceinline__ void write(long long wid, const trk::TrackResult& R) const {
+    a.status[wid] = (uint8_t)R.status;
+    if (a.out3) {
+      a.out3[3 * wid] = R.x;
+      a.out3[3 * wid + 1] = R.y;
+      a.out3[3 * wid + 2] = R.th;
+    }
+    if (a.out2) {
+      a.out2[2 * wid] = R.x;
+      a.out2[2 * wid + 1] = R.y;
+    }
+    if (a.fb_dist) a.fb_dist[wid] = R.dist;
+    if (a.last_step) a.last_step[wid] = R.last;
+  }
+};
+
+__global__ void __launch_bounds__(trk::kGroupThreads, trk::kGroupCtasPerSm)
+    track_groups_kernel(const __grid_constant__ TrackArgs a) {
+  constexpr int WPB = trk::kGroupThreads / 32;
+  __shared__ __align__(16) uint8_t smem[WPB * trk::kWarpBytes<trk::kGroupLanes>];
+  const int warp = threadIdx.x >> 5;
+  trk::run_tracks<trk::kGroupLanes>(StageSource{a}, (long long)blockIdx.x * WPB + warp,
+                                    (long long)gridDim.x * WPB,
+                                    smem + warp * trk::kWarpBytes<trk::kGroupLanes>);
+}
+
 __global__ void fb_check_kernel(const float* __restrict__ orig, const float* __restrict__ back,
                                 const int32_t* __restrict__ count, int capacity,
                                 long long total, float max_dist, uint8_t* __restrict__ status,
@@ -98,6 +172,12 @@ cudaError_t launch_track(const Geom& g, const Batch& src, const Batch& dst, cons
               shared_pts ? 1 : 0};
   const long long warps = (long long)capacity * src.n;
   if (warps == 0) return cudaSuccess;
+  // a warp per keypoint while they leave much of the GPU idle (a warp is done
+  // sooner), groups of lanes beyond (track_group.cuh has both sides measured)
+  if (warps >= 28LL * sm_count()) {
+    track_groups_kernel<<<(unsigned)trk::group_ctas(warps), trk::kGroupThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   const long long blocks = (warps * 32 + TRK_THREADS - 1) / TRK_THREADS;
   track_kernel<<<(unsigned)blocks, TRK_THREADS, 0, s>>>(a);
   return cudaGetLastError();
