@@ -511,9 +511,10 @@ vio_status vio_frontend_set_initnet(vio_frontend* fe, const void* d_packed,
 /* --------------------------------------------------------------- batch -- */
 /* Many stereo streams of mixed sizes in one step (the frontend of Sec. III-B
  * for each stream; batching streams is not in the paper). Streams are
- * grouped by size (up to 8 groups); every step runs the same three launches
- * for all groups (one per stage), optionally replayed from a captured CUDA
- * graph. Each stream keeps its own state on the device: its two frame
+ * grouped by size (up to 8 groups); every step runs the same launches
+ * for all groups (one per stage; the front of a step of 4 Mi pixels or more:
+ * one per pyramid level and one for the detection), optionally replayed from
+ * a captured CUDA graph. Each stream keeps its own state on the device: its two frame
  * slots, keypoint lists, ids and first-frame flag; a step advances only the
  * streams marked active, the others keep their state untouched. */
 typedef struct vio_batch vio_batch;
@@ -526,15 +527,18 @@ typedef struct {
 } vio_stream_group;
 
 /* Tunables of a batch step: threads per block of the tracking launches (32,
- * 64, 128, 256 or 512; one warp tracks one keypoint, so small blocks spread
- * the warps evenly over the SMs), the pyramid tile scale (-1, 0, 1: half, default, double
+ * 64, 128, 256 or 512) where one warp tracks one keypoint (steps of 10 to 46
+ * keypoint slots per SM, and the stereo matching after selection; smaller
+ * steps give a keypoint two warps, larger ones four lanes, each at a block
+ * size of its own), the pyramid tile scale (-1, 0, 1: half, default, double
  * the deepest-level tile side), the order of stereo matching (0: every
  * cell's candidates are matched beside temporal tracking; 1: only the
  * selected keypoints are matched, after selection, in two more launches),
  * the pyramid levels the fused pyramid+detection launch computes (1..4,
- * 0 = up to 4; the rest follow in further pyramid launches: fewer levels per
- * pass recompute less of the halo of level 0), the CTA size of that launch
- * (128 or 256) and the warps that score one detection cell (1, 2, 4 or 8, at
+ * 0 = up to 4, or one launch per level and the detection alone for a step of
+ * 4 Mi pixels or more; the rest follow in further pyramid launches: fewer
+ * levels per pass recompute less of the halo of level 0), the CTA size of the
+ * fused launch (128 or 256) and the warps that score one detection cell (1, 2, 4 or 8, at
  * most CTA size / 32; 0 = chosen from the launch: one when its cells fill the
  * GPU, more for few cells). Every setting gives the same lists bit for bit. */
 typedef struct vio_batch_tune_s {

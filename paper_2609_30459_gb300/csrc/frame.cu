@@ -6,17 +6,22 @@
 //                           (one pyramid pass per tile) and, in the same
 //                           launch, the per-cell FAST/NMS top-k candidates of
 //                           camera 0. Levels beyond 4 follow as a further pass.
+//                           A large step runs frame_level_kernel per level and
+//                           K1 for the detection alone (split_front).
 //  KN frame_initnet_kernel  (only with the learned initializer) persistent
 //                           CTAs over rounds of 32 live tracks of one
 //                           camera: network input from the previous and
 //                           current pyramids, forward pass on the tcgen05
 //                           tensor cores -> flow proposal + confidence.
-//  K2 frame_track_kernel    one warp per keypoint: temporal tracking of every
-//                           live track of both cameras (previous -> current
-//                           pyramid; from the proposal over the lower levels
-//                           when it is confident, the plain track otherwise
-//                           or when that fails) AND stereo matching (camera 0
-//                           -> 1) of every cell's top-k candidates.
+//  K2 frame_track_kernel    one warp per keypoint (two in a small step,
+//                           frame_track_team_kernel; four lanes in a large
+//                           one, frame_track_groups_kernel): temporal
+//                           tracking of every live track of both cameras
+//                           (previous -> current pyramid; from the proposal
+//                           over the lower levels when it is confident, the
+//                           plain track otherwise or when that fails) AND
+//                           stereo matching (camera 0 -> 1) of every cell's
+//                           top-k candidates.
 //  K3 frame_finalize_kernel one CTA per stream: keep the tracks that passed,
 //                           count them per cell, select per cell the first
 //                           k - count candidates (the detection of Sec. III-D
@@ -46,7 +51,7 @@
 #include "initnet_dev.cuh"
 #include "initnet_tc.cuh"
 #include "pyramid_dev.cuh"
-#include "track_group.cuh"
+#include "track_team.cuh"
 
 namespace vio {
 namespace {
@@ -334,9 +339,6 @@ __global__ void __launch_bounds__(ntc::THREADS, 1) frame_initnet_kernel(
 #define VIO_TRACK_BOUNDS
 #endif
 
-// BUTTERFLY: the reduction form for a launch that leaves most of the GPU
-// idle (trk::warp_sum4).
-template <bool BUTTERFLY>
 __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ MultiK2 mm) {
   // the finalisation (launched as this launch's programmatic dependent) may
   // take its SM now and wait there for this launch's completion
@@ -374,7 +376,7 @@ __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ Mult
       const float* q = f.net_out + 3 * wl;
       if (q[2] >= f.net_tau) {
         float last;
-        st = trk::track_fb<BUTTERFLY>(f.g, f.prev, r.prev_img + c, f.cur, r.cur_img + c, px, py,
+        st = trk::track_fb(f.g, f.prev, r.prev_img + c, f.cur, r.cur_img + c, px, py,
                                       true, px + q[0], py + q[1], 0.f, cfg, f.net_top, lane, tf,
                                       thf, have, dist, last);
         learned = st == VIO_TRACK_OK && !(f.net_max_step > 0.f && last > f.net_max_step);
@@ -382,7 +384,7 @@ __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ Mult
     }
     if (!learned) {
       float last;
-      st = trk::track_fb<BUTTERFLY>(f.g, f.prev, r.prev_img + c, f.cur, r.cur_img + c, px, py,
+      st = trk::track_fb(f.g, f.prev, r.prev_img + c, f.cur, r.cur_img + c, px, py,
                                     false, 0.f, 0.f, 0.f, cfg, top, lane, tf, thf, have, dist,
                                     last);
     }
@@ -411,7 +413,7 @@ __global__ void VIO_TRACK_BOUNDS frame_track_kernel(const __grid_constant__ Mult
   const unsigned idx = ~(unsigned)(key & 0xffffffffu);
   const float x = (float)(idx % (unsigned)f.g.w[0]), y = (float)(idx / (unsigned)f.g.w[0]);
   float last;
-  const int st = trk::track_fb<BUTTERFLY>(f.g, f.cur, r.cur_img, f.cur, r.cur_img + 1, x, y,
+  const int st = trk::track_fb(f.g, f.cur, r.cur_img, f.cur, r.cur_img + 1, x, y,
                                           false, 0.f, 0.f, 0.f, cfg, top, lane, tf, thf, have,
                                           dist, last);
   if (lane == 0) {
@@ -539,6 +541,14 @@ __global__ void __launch_bounds__(trk::kGroupThreads, trk::kGroupCtasPerSm)
   trk::run_tracks<trk::kGroupLanes>(FrameTracks{mm}, (long long)blockIdx.x * WPB + warp,
                                     (long long)gridDim.x * WPB,
                                     smem + warp * trk::kWarpBytes<trk::kGroupLanes>);
+}
+
+// A CTA per slot.
+__global__ void __launch_bounds__(trk::kTeamThreads, trk::kTeamCtasPerSm)
+    frame_track_team_kernel(const __grid_constant__ MultiK2 mm) {
+  asm volatile("griddepcontrol.launch_dependents;");   // as in frame_track_kernel
+  __shared__ trk::TeamSmem sm;
+  trk::team_track(FrameTracks{mm}, blockIdx.x, sm);
 }
 
 struct MultiK3 {
@@ -894,10 +904,10 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     const long long blocks2 = (acc * 32 + k2t - 1) / k2t;
     if (acc >= kGroupSlotsPerSm * sm_count())
       frame_track_groups_kernel<<<(unsigned)trk::group_ctas(acc), trk::kGroupThreads, 0, s>>>(m2);
-    else if (k2_small)
-      frame_track_kernel<true><<<(unsigned)blocks2, k2t, 0, s>>>(m2);
+    else if (acc <= trk::team_ctas())   // one wave (track_team.cuh)
+      frame_track_team_kernel<<<(unsigned)acc, trk::kTeamThreads, 0, s>>>(m2);
     else
-      frame_track_kernel<false><<<(unsigned)blocks2, k2t, 0, s>>>(m2);
+      frame_track_kernel<<<(unsigned)blocks2, k2t, 0, s>>>(m2);
   }
 
   // K3: finalize

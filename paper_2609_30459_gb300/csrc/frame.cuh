@@ -9,7 +9,7 @@ constexpr int kMaxGroups = 8;
 
 // Launch tunables (chosen by the autotuner of a batch).
 struct FrameTune {
-  int k2_threads;      // threads per block of the tracking launch (64..512)
+  int k2_threads;      // threads per block where a warp tracks a keypoint (32..512)
   int pyr_tile_shift;  // deepest-level pyramid tile side = (32 >> (m-1)) << shift
   int stereo_after;    // 1: stereo-match only the selected keypoints, after selection
   int pyr_first;       // pyramid levels of K1's fused pass (1..4; 0 = as many as fit)

@@ -1,8 +1,9 @@
 // Pyramidal inverse-compositional KLT (Sec. III-E, Eq. 4-5) for the stage
 // entry points vio_track_patches / vio_stereo_match, and the
 // forward-backward distance check. The tracker itself is in track_dev.cuh (a
-// warp per keypoint) and track_group.cuh (large launches).
-#include "track_group.cuh"
+// warp per keypoint), track_team.cuh (small launches) and track_group.cuh
+// (large ones).
+#include "track_team.cuh"
 
 namespace vio {
 namespace {
@@ -144,6 +145,13 @@ __global__ void __launch_bounds__(trk::kGroupThreads, trk::kGroupCtasPerSm)
                                     smem + warp * trk::kWarpBytes<trk::kGroupLanes>);
 }
 
+// A CTA per keypoint.
+__global__ void __launch_bounds__(trk::kTeamThreads, trk::kTeamCtasPerSm)
+    track_team_kernel(const __grid_constant__ TrackArgs a) {
+  __shared__ trk::TeamSmem sm;
+  trk::team_track(StageSource{a}, blockIdx.x, sm);
+}
+
 __global__ void fb_check_kernel(const float* __restrict__ orig, const float* __restrict__ back,
                                 const int32_t* __restrict__ count, int capacity,
                                 long long total, float max_dist, uint8_t* __restrict__ status,
@@ -172,10 +180,15 @@ cudaError_t launch_track(const Geom& g, const Batch& src, const Batch& dst, cons
               shared_pts ? 1 : 0};
   const long long warps = (long long)capacity * src.n;
   if (warps == 0) return cudaSuccess;
-  // a warp per keypoint while they leave much of the GPU idle (a warp is done
-  // sooner), groups of lanes beyond (track_group.cuh has both sides measured)
+  // groups of lanes where the keypoints fill the GPU, a warp each where they
+  // are fewer (track_group.cuh has both sides measured)
   if (warps >= 28LL * sm_count()) {
     track_groups_kernel<<<(unsigned)trk::group_ctas(warps), trk::kGroupThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
+  // one wave of CTAs of two warps each (track_team.cuh)
+  if (warps <= trk::team_ctas()) {
+    track_team_kernel<<<(unsigned)warps, trk::kTeamThreads, 0, s>>>(a);
     return cudaGetLastError();
   }
   const long long blocks = (warps * 32 + TRK_THREADS - 1) / TRK_THREADS;

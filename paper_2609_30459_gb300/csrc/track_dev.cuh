@@ -106,6 +106,28 @@ __device__ __forceinline__ LanePts lane_points(int lane) {
   return P;
 }
 
+// Two values at a time, as the two lanes of packed FP32 instructions: the same
+// IEEE operation on each half.
+#ifdef __CUDACC__
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) { return __fadd2_rd(a, b); }
+#else
+inline float2 fma2(float2 a, float2 b, float2 c) {
+  return float2{__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y)};
+}
+inline float2 add2(float2 a, float2 b) { return float2{a.x + b.x, a.y + b.y}; }
+inline float2 mul2(float2 a, float2 b) {
+  return float2{__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y)};
+}
+inline float2 add2_rd(float2 a, float2 b) {
+  return float2{__fadd_rd(a.x, b.x), __fadd_rd(a.y, b.y)};
+}
+#endif
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.f), a); }
+
 struct Lv {
   const uint8_t* p;
   int w, h, pitch;
@@ -119,31 +141,13 @@ __device__ __forceinline__ void warp_sum(float (&v)[N]) {
     for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
 }
 
-// Sums four values over the warp and gives every lane all four totals.
-// BUTTERFLY: an xor butterfly, five rounds of four independent exchanges
-// (the two lanes of every exchange add the same two operands, so partners
-// hold bitwise equal partial sums after each round and every lane ends with
-// the same totals): the shortest dependent chain, for launches that leave the
-// GPU mostly idle. Else a transposed butterfly with half the exchanges (after
-// the xor-16 and xor-8 rounds each lane carries one of the four partial sums,
-// value 2*bit4 + bit3 of its lane id, three more xor rounds finish it, four
-// broadcasts hand it out): fewer instructions, for launches that fill it.
-template <bool BUTTERFLY>
+// Sums four values over the warp and gives every lane all four totals, by a
+// transposed butterfly: after the xor-16 and xor-8 rounds each lane carries one
+// of the four partial sums (value 2*bit4 + bit3 of its lane id), three more xor
+// rounds finish it, four broadcasts hand it out. Half the exchanges of a plain
+// butterfly, and the shorter wait too: four tracks of an SM finished after
+// 18.1 us with this form and 19.0 us with that one.
 __device__ __forceinline__ void warp_sum4(float& a0, float& a1, float& a2, float& a3) {
-  if (BUTTERFLY) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float b0 = __shfl_xor_sync(0xffffffffu, a0, o);
-      const float b1 = __shfl_xor_sync(0xffffffffu, a1, o);
-      const float b2 = __shfl_xor_sync(0xffffffffu, a2, o);
-      const float b3 = __shfl_xor_sync(0xffffffffu, a3, o);
-      a0 += b0;
-      a1 += b1;
-      a2 += b2;
-      a3 += b3;
-    }
-    return;
-  }
   const unsigned lane = threadIdx.x & 31u;
   const bool h16 = lane & 16u, h8 = lane & 8u;
   float k0 = h16 ? a2 : a0, k1 = h16 ? a3 : a1;
@@ -365,46 +369,52 @@ constexpr float kPatRadius = 7.6158f;
 
 // One Gauss-Newton step (Eq. 4-5). Returns a VIO_TRACK_* status; `moved` is
 // the bound above on how far the step moved the pattern (level px).
-template <bool BUTTERFLY = false>
 __device__ __forceinline__ int gn_step(const Lv& L, const Tpl& T, int lane, const LanePts& P,
                                        Warp& W, float& moved) {
-  float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f;
   bool ok = true;
   const unsigned xmax = (unsigned)(L.w - 2), ymax = (unsigned)(L.h - 2);
-  // no branch in the loop: a lane without a second point evaluates the
-  // pattern's centre with weight 0 (its K is 0 too); it lies inside the
-  // level whenever the pattern's points do. A sample outside the level is
-  // read at the clamped position and only clears `ok`.
+  // the lane's two points side by side, no branch: a lane without a second
+  // point evaluates the pattern's centre with weight 0 (its K is 0 too); it
+  // lies inside the level whenever the pattern's points do. A sample outside
+  // the level is read at the clamped position and only clears `ok`.
+  const float2 u = make_float2(P.u[0], P.u[1]), v = make_float2(P.v[0], P.v[1]);
+  const float2 vx = fma2(both(W.cs), u, fma2(both(-W.sn), v, both(W.t.dx)));
+  const float2 vy = fma2(both(W.sn), u, fma2(both(W.cs), v, both(W.t.dy)));
+  // floor without a conversion instruction: adding 1.5 * 2^23 rounded down
+  // leaves floor(v) in the low mantissa bits (exact for |v| < 2^22; beyond
+  // that the sample is outside the level either way)
+  const float2 tx = add2_rd(vx, both(kFloorBias)), ty = add2_rd(vy, both(kFloorBias));
+  const float2 fx = sub2(vx, add2(tx, both(-kFloorBias)));
+  const float2 fy = sub2(vy, add2(ty, both(-kFloorBias)));
+  float px[2][4];
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
-    const float u = P.u[j], v = P.v[j];
-    const float vx = __fmaf_rn(W.cs, u, __fmaf_rn(-W.sn, v, W.t.dx));
-    const float vy = __fmaf_rn(W.sn, u, __fmaf_rn(W.cs, v, W.t.dy));
-    // floor without a conversion instruction: adding 1.5 * 2^23 rounded
-    // down leaves floor(v) in the low mantissa bits (exact for |v| < 2^22;
-    // beyond that the sample is outside the level either way)
-    const float tx = __fadd_rd(vx, kFloorBias), ty = __fadd_rd(vy, kFloorBias);
-    const int ix = W.t.ax + (__float_as_int(tx) - kFloorBiasBits);
-    const int iy = W.t.ay + (__float_as_int(ty) - kFloorBiasBits);
-    const float fx = vx - (tx - kFloorBias), fy = vy - (ty - kFloorBias);
+    const int ix = W.t.ax + (__float_as_int(j ? tx.y : tx.x) - kFloorBiasBits);
+    const int iy = W.t.ay + (__float_as_int(j ? ty.y : ty.x) - kFloorBiasBits);
     // 0 <= y < w - 1 on the integer part: 0 <= ix <= w - 2 (one unsigned test)
     ok = ok && (unsigned)ix <= xmax && (unsigned)iy <= ymax;
     const unsigned cx = min((unsigned)ix, xmax), cy = min((unsigned)iy, ymax);
     const uint8_t* p = L.p + (cy * (unsigned)L.pitch + cx);
-    const float a = __ldg(p), b = __ldg(p + 1);
-    const float c = __ldg(p + L.pitch), d = __ldg(p + L.pitch + 1);
-    const float top = __fmaf_rn(fx, b - a, a), bot = __fmaf_rn(fx, d - c, c);
-    const float r = __fmaf_rn(fy, bot - top, top);
-    r0 = j == 0 ? r0 + r : __fmaf_rn(P.w1, r, r0);
-    r1 = __fmaf_rn(T.K[j][0], r, r1);
-    r2 = __fmaf_rn(T.K[j][1], r, r2);
-    r3 = __fmaf_rn(T.K[j][2], r, r3);
+    px[j][0] = __ldg(p);
+    px[j][1] = __ldg(p + 1);
+    px[j][2] = __ldg(p + L.pitch);
+    px[j][3] = __ldg(p + L.pitch + 1);
   }
+  const float2 a = make_float2(px[0][0], px[1][0]), b = make_float2(px[0][1], px[1][1]);
+  const float2 c = make_float2(px[0][2], px[1][2]), d = make_float2(px[0][3], px[1][3]);
+  const float2 top = fma2(fx, sub2(b, a), a), bot = fma2(fx, sub2(d, c), c);
+  const float2 r = fma2(fy, sub2(bot, top), top);
+  const float2 zero = both(0.f);
+  const float2 r03 = fma2(make_float2(P.w1, T.K[1][2]), both(r.y),
+                          fma2(make_float2(1.f, T.K[0][2]), both(r.x), zero));
+  const float2 r12 = fma2(make_float2(T.K[1][0], T.K[1][1]), both(r.y),
+                          fma2(make_float2(T.K[0][0], T.K[0][1]), both(r.x), zero));
+  float r0 = r03.x, r1 = r12.x, r2 = r12.y, r3 = r03.y;
   // a sample outside the level adds 1e30 to the sum of intensities (at most
   // 52 x 255 otherwise), so the one reduction also tells every lane whether
   // any lane left the level
   if (!ok) r0 += 1e30f;
-  warp_sum4<BUTTERFLY>(r0, r1, r2, r3);
+  warp_sum4(r0, r1, r2, r3);
   // the increment before its checks, so that one branch takes all three
   // failures (in this order): a sample outside the level, a non-positive
   // mean, a non-finite increment (a NaN or an infinity in any component
@@ -418,12 +428,12 @@ __device__ __forceinline__ int gn_step(const Lv& L, const Tpl& T, int lane, cons
     return r0 >= 1e29f ? VIO_TRACK_OOB_WARP : !(r0 > 0.f) ? VIO_TRACK_ZERO_MEAN : VIO_TRACK_NAN;
   moved = __fmaf_rn(kPatRadius, fabsf(d2), s01);
   // T <- T o exp(delta): t += R V(d2) (d0, d1), R <- R R(d2)
-  float cd, sd, a, b;
-  small_rot(d2, cd, sd, a, b);
-  const float vx = __fmaf_rn(-b, d1, __fmul_rn(a, d0));
-  const float vy = __fmaf_rn(a, d1, __fmul_rn(b, d0));
-  W.t.dx = __fmaf_rn(W.cs, vx, __fmaf_rn(-W.sn, vy, W.t.dx));
-  W.t.dy = __fmaf_rn(W.sn, vx, __fmaf_rn(W.cs, vy, W.t.dy));
+  float cd, sd, va, vb;
+  small_rot(d2, cd, sd, va, vb);
+  const float mx = __fmaf_rn(-vb, d1, __fmul_rn(va, d0));
+  const float my = __fmaf_rn(va, d1, __fmul_rn(vb, d0));
+  W.t.dx = __fmaf_rn(W.cs, mx, __fmaf_rn(-W.sn, my, W.t.dx));
+  W.t.dy = __fmaf_rn(W.sn, mx, __fmaf_rn(W.cs, my, W.t.dy));
   const float cs = __fmaf_rn(-W.sn, sd, __fmul_rn(W.cs, cd));
   const float sn = __fmaf_rn(W.cs, sd, __fmul_rn(W.sn, cd));
   W.cs = cs;
@@ -442,7 +452,6 @@ __device__ __forceinline__ Lv get_lv(const Geom& g, const Batch& b, int img, int
 // level whose template is invalid is skipped, except level 0; any warp
 // failure ends the track. last_step: how far the last Gauss-Newton step at
 // level 0 moved the pattern (bound of gn_step, level-0 px; 0 if none ran).
-template <bool BUTTERFLY = false>
 __device__ __forceinline__ int track_dir(const Geom& g, const Batch& src, int src_img,
                                          const Batch& dst, int dst_img, const Pos& p, Pos t0,
                                          float th0, int iters, int top, int lane, Pos& t_out,
@@ -466,7 +475,7 @@ __device__ __forceinline__ int track_dir(const Geom& g, const Batch& src, int sr
       const Lv D = get_lv(g, dst, dst_img, l);
       float moved = 0.f;
       for (int it = 0; it < iters; ++it) {
-        const int st = gn_step<BUTTERFLY>(D, T, lane, P, W, moved);
+        const int st = gn_step(D, T, lane, P, W, moved);
         if (st != VIO_TRACK_OK) return st;
       }
       if (l == 0) last_step = moved;
@@ -489,7 +498,6 @@ __device__ __forceinline__ int track_dir(const Geom& g, const Batch& src, int sr
 // over levels top..0, from warp (ix, iy, ith) if has_init, else from p.
 // Returns the status; tf/thf hold the forward result when it exists and
 // last_fwd the forward pass's last level-0 step (track_dir).
-template <bool BUTTERFLY = false>
 __device__ __forceinline__ int track_fb(const Geom& g, const Batch& src, int src_img,
                                         const Batch& dst, int dst_img, float px, float py,
                                         bool has_init, float ix, float iy, float ith,
@@ -502,7 +510,7 @@ __device__ __forceinline__ int track_fb(const Geom& g, const Batch& src, int src
     t0 = split(ix, iy);
     th0 = ith;
   }
-  int st = track_dir<BUTTERFLY>(g, src, src_img, dst, dst_img, p, t0, th0, cfg.gn_iters, top,
+  int st = track_dir(g, src, src_img, dst, dst_img, p, t0, th0, cfg.gn_iters, top,
                                 lane, tf, thf, last_fwd);
   have = st == VIO_TRACK_OK;
   dist = __int_as_float(0x7fc00000);
@@ -511,7 +519,7 @@ __device__ __forceinline__ int track_fb(const Geom& g, const Batch& src, int src
     // start at the forward estimate's inverse (t = p, theta = -theta_f)
     Pos tb;
     float thb, last_b;
-    st = track_dir<BUTTERFLY>(g, dst, dst_img, src, src_img, tf, p, -thf, cfg.gn_iters, top,
+    st = track_dir(g, dst, dst_img, src, src_img, tf, p, -thf, cfg.gn_iters, top,
                               lane, tb, thb, last_b);
     if (st == VIO_TRACK_OK) {
       const float ex = (float)(tb.ax - p.ax) + (tb.dx - p.dx);

@@ -53,16 +53,6 @@ static_assert(kWinCols + 4 <= 32 && kTplCols + 4 <= 32 && kPitch >= 32 && kGroup
               "a region's columns fit its rows, groups start four banks apart");
 constexpr float kReach = 7.63f;   // > radius of the pattern, with room for rounding
 
-// Two samples of a lane at a time, as the two lanes of packed FP32
-// instructions (half the issue slots; each lane rounds as the scalar
-// instruction does).
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2_rd(float2 a, float2 b) { return __fadd2_rd(a, b); }
-__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.f), a); }
-
 // Lane gl of a group owns the pattern points gl + LPK s, slot s < 2 NP, in
 // pairs of slots (2 j, 2 j + 1). A slot without a point has weight 0 (and
 // K = 0) and stands at the pattern's centre; only the last pair has any.
