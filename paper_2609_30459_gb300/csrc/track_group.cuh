@@ -20,10 +20,12 @@
 //
 // Measured (640 x 480, five levels, five steps, forward and backward, us;
 // keypoints: one per warp / 4 lanes / 8 lanes each):
-//   2400: 41 / 57 / 43    4800: 68 / 57 / 51    9600: 112 / 70 / 78
-//   14400: 158 / 96 / 129    24000: 246 / 185 / 234
-// A group of four lanes takes about 55 us however few keypoints there are, so a
-// launch of fewer than 28 keypoints per SM keeps a warp each.
+//   2400: 38 / 57 / 43    4200: 57 / 57    4800: 68 / 57 / 51
+//   9600: 112 / 70 / 78   14400: 158 / 96 / 129    24000: 246 / 185 / 234
+// (one per warp: 2400 and 4200 with the packed step of track_dev.cuh, the
+// others before it). A group of four lanes takes about 55 us however few
+// keypoints there are, so a launch of fewer than 28 keypoints per SM keeps a
+// warp each.
 //
 // A group is a small state machine (keypoint, direction, level) that advances
 // by one level per turn of the warp's loop, independently of the warp's other
