@@ -46,15 +46,15 @@ CONFIG = {"workload": WORKLOAD, "frames": N_FRAMES, "w": W, "h": H, "levels": LE
 # algorithmic FP32 operations of one keypoint through one direction at one
 # level of the KLT: template 52 x ~72 + 5 Gauss-Newton steps of 52 x ~26
 FLOPS_PER_KP_DIR_LEVEL = 52 * 72 + 5 * 52 * 26
-# ncu counters of frame_track_kernel on this workload (the profile summary in
+# ncu counters of the tracking launch on this workload (the profile summary in
 # profiles/ names the command)
-TRACK_NCU = {"profile": "profiles/frame_kernels_752x480.md"}
+TRACK_NCU = {"profile": "profiles/tracking_launches.md"}
 # DRAM bytes (read + write) per image of the pyramid+detection pass
-# (vio_pyramid_detect: pyr_pass_kernel, detect_cells_kernel, select_kernel),
+# (vio_pyramid_detect: pyr_level_kernel, detect_cells_kernel, select_kernel),
 # from an ncu capture of 512 images of the headline sequence with the L2 kept
 # between launches (profiles/pyramid_detect_752x480x512.md names the command);
 # a full launch moves this per image
-PYRDET_TRAFFIC_PER_IMAGE = 808243
+PYRDET_TRAFFIC_PER_IMAGE = 694718
 
 
 def seq_seed(rank: int) -> int:
@@ -371,13 +371,13 @@ def pyramid_detect_roofline(torch, vio, frames_dev, peaks, peak_src, w=None, h=N
             "traffic_note": "DRAM read + write bytes per launch: an ncu capture of 512 images (L2 kept "
                             "between launches) "
                             "scaled by the images of this launch",
-            "kernel": "vio_pyramid_detect (pyr_pass_kernel, detect_cells_kernel, select_kernel)",
+            "kernel": "vio_pyramid_detect (pyr_level_kernel, detect_cells_kernel, select_kernel)",
             "images": n, "image": f"{w}x{h}, {levels} levels, {gx}x{gy} cells",
             "batch_bytes_in": n * w * h, "algorithmic_bytes": alg,
             "algorithmic_bytes_per_image": w * h + upper + n_kp * 10 / n,
             "ms": 1000 * t, "peak_source": peak_src,
             "note": "vio_pyramid_detect: per chunk of images (level 0 at most 64 MiB) the "
-                    "pyramid launch (levels 1-2, then 3) and the per-cell FAST/NMS/top-k "
+                    "pyramid launches (one per level) and the per-cell FAST/NMS/top-k "
                     "launch, then the per-image selection; algorithmic bytes: level 0 read "
                     "once, upper levels and 10 B per keypoint written"}
 
@@ -1166,7 +1166,7 @@ def main():
     # its launch time, with the issue and stall counters of its ncu profile
     per_stage = {k: v / max(n_timed, 1) for k, v in stage_ms.items()}
     t_track = stage_ms["track"] / 1000.0 / max(n_timed, 1)
-    tracking = {"kernel": "frame_track_kernel",
+    tracking = {"kernel": "frame_track_team_kernel",
                 "keypoints_per_launch": (tracked + stereo_in) / args.steps,
                 "keypoint_tracks_per_s": (tracked + stereo_in) / args.steps / t_track,
                 "avg_launch_us": 1e6 * t_track,
