@@ -527,7 +527,7 @@ typedef struct {
 } vio_stream_group;
 
 /* Tunables of a batch step: threads per block of the tracking launches (32,
- * 64, 128, 256 or 512) where one warp tracks one keypoint (steps of 10 to 46
+ * 64, 128, 256 or 512) where one warp tracks one keypoint (steps of 10 to 200
  * keypoint slots per SM, and the stereo matching after selection; smaller
  * steps give a keypoint two warps, larger ones four lanes, each at a block
  * size of its own), the pyramid tile scale (-1, 0, 1: half, default, double

@@ -691,9 +691,12 @@ bool split_front(const Geom* g, const int* n_streams, int n_groups, int pyr_firs
 }
 
 // Slots of a step's tracking launch per SM from which it runs by groups of lanes
-// (track_group.cuh) instead of a warp per keypoint: 28 keypoints, and about
-// three in five slots of a step hold one.
-constexpr long long kGroupSlotsPerSm = 46;
+// (track_group.cuh) instead of a warp per keypoint. Many slots of a step are
+// empty and many tracks end early, which costs a warp of its own little and a
+// group its turn: plain and learned steps of mixed batches took, groups / warps,
+// 524 / 413 us at 63 slots per SM (four steps), 323 / 253 at 139, 333 / 259 at
+// 154, 418 / 328 at 179.
+constexpr long long kGroupSlotsPerSm = 200;
 
 // Levels the fused pass of K1 computes (the rest follow in further passes);
 // pyr_first < 0: none.

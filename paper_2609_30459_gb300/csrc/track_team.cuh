@@ -54,9 +54,8 @@ __device__ __forceinline__ void touch_target(const Lv& D, const Pos& t, int l, c
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int x = min(max(qx + P.iu[j], 0), D.w - 1), y = min(max(qy + P.iv[j], 0), D.h - 1);
-    unsigned v;
-    asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(v) : "l"(D.p + (long long)y * D.pitch + x));
-    (void)v;
+    unsigned v = 0;
+    asm volatile("ld.global.nc.u8 %0, [%1];" : "+r"(v) : "l"(D.p + (long long)y * D.pitch + x));
   }
 #endif
 }
