@@ -181,8 +181,12 @@ cudaError_t launch_track(const Geom& g, const Batch& src, const Batch& dst, cons
   const long long warps = (long long)capacity * src.n;
   if (warps == 0) return cudaSuccess;
   // groups of lanes where the keypoints fill the GPU, a warp each where they
-  // are fewer (track_group.cuh has both sides measured)
-  if (warps >= 28LL * sm_count()) {
+  // are fewer; rows that start at any byte cost a group more (track_group.cuh
+  // has both sides measured for either)
+  const bool words =
+      ((reinterpret_cast<uintptr_t>(src.l0) | reinterpret_cast<uintptr_t>(dst.l0) |
+        (uintptr_t)src.l0_stride | (uintptr_t)dst.l0_stride | (uintptr_t)g.pitch[0]) & 3) == 0;
+  if (warps >= (words ? 28LL : 48LL) * sm_count()) {
     track_groups_kernel<<<(unsigned)trk::group_ctas(warps), trk::kGroupThreads, 0, s>>>(a);
     return cudaGetLastError();
   }

@@ -26,6 +26,12 @@
 // others before it). A group of four lanes takes about 55 us however few
 // keypoints there are, so a launch of fewer than 28 keypoints per SM keeps a
 // warp each.
+// Level-0 rows that start at any byte (641 x 479; one per warp / 4 lanes, and in
+// brackets 4 lanes copying such rows byte by byte, as they first did):
+//   9280: 108 / 79 (102)    23200: 236 / 216 (288)
+//   level 0 alone: 9280: 34 / 27 (52)    23200: 70 / 62 (105)
+//   753 x 481, 6216: 78 / 76 (106)    level 0 alone: 22.9 / 24.0 (49.6)
+// so such launches keep a warp each below 48 keypoints per SM.
 //
 // A group is a small state machine (keypoint, direction, level) that advances
 // by one level per turn of the warp's loop, independently of the warp's other
@@ -150,25 +156,45 @@ __device__ __forceinline__ void copy_region(uint8_t* dst, const Lv& L, int x0, i
     }
     return;
   }
-  // a word (or byte) at a time
+  if ((al & 3) == 0) {
+    // a word at a time
 #pragma unroll 1
-  for (int s = gl; s < COLS / 4; s += LPK) {
-    const int x = x0 + 4 * s;
-    if (x < 0 || x >= L.w) continue;
-    uint8_t* d = dst + (x0 & 7) + 4 * s;
+    for (int s = gl; s < COLS / 4; s += LPK) {
+      const int x = x0 + 4 * s;
+      if (x < 0 || x >= L.w) continue;
+      uint8_t* d = dst + (x0 & 7) + 4 * s;
 #pragma unroll 6
-    for (int r = 0; r < ROWS; ++r) {
-      const int y = min(max(y0 + r, 0), L.h - 1);
-      const uint8_t* p = L.p + ((unsigned)y * (unsigned)L.pitch + (unsigned)x);
-      if ((al & 3) == 0) {
-        __pipeline_memcpy_async(d + r * kPitch, p, 4);
-      } else {
-        unsigned v = 0u;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          if (x + b < L.w) v |= (unsigned)__ldg(p + b) << (8 * b);
-        *reinterpret_cast<unsigned*>(d + r * kPitch) = v;
+      for (int r = 0; r < ROWS; ++r) {
+        const int y = min(max(y0 + r, 0), L.h - 1);
+        __pipeline_memcpy_async(d + r * kPitch,
+                                L.p + ((unsigned)y * (unsigned)L.pitch + (unsigned)x), 4);
       }
+    }
+    return;
+  }
+  // rows that start at any byte: a row per lane, aligned words shifted into
+  // place; bytes where such a word might lie outside the image
+  constexpr int NW = COLS / 4;
+  const uintptr_t begin = reinterpret_cast<uintptr_t>(L.p);
+  const uintptr_t end = begin + (unsigned)(L.h - 1) * (unsigned)L.pitch + (unsigned)L.w;
+#pragma unroll 3
+  for (int r = gl; r < ROWS; r += LPK) {
+    const int y = min(max(y0 + r, 0), L.h - 1);
+    const uint8_t* row = L.p + (unsigned)y * (unsigned)L.pitch;
+    uint8_t* d = dst + (r * kPitch + (x0 & 7));
+    const uintptr_t p = reinterpret_cast<uintptr_t>(row) + (intptr_t)x0, a = p & ~(uintptr_t)3;
+    if (a >= begin && a + 4 * (NW + 1) <= end) {
+      const unsigned* q = reinterpret_cast<const unsigned*>(a);
+      const int sh = 8 * (int)(p & 3);
+      unsigned w[NW + 1];
+#pragma unroll
+      for (int k = 0; k <= NW; ++k) w[k] = __ldg(q + k);
+#pragma unroll
+      for (int k = 0; k < NW; ++k)
+        *reinterpret_cast<unsigned*>(d + 4 * k) = __funnelshift_r(w[k], w[k + 1], sh);
+    } else {
+#pragma unroll 1
+      for (int x = max(x0, 0); x < min(x0 + COLS, L.w); ++x) d[x - x0] = __ldg(row + x);
     }
   }
 }
