@@ -59,7 +59,10 @@ constexpr int kGroupBytes = kTplBytes + kWinRows * kPitch;
 static_assert(kWinCols + 4 <= 32 && kTplCols + 4 <= 32 && kPitch >= 32 && kGroupBytes % 16 == 0 &&
                   kGroupBytes / 4 % 32 == 4,
               "a region's columns fit its rows, groups start four banks apart");
-constexpr float kReach = 7.63f;   // > radius of the pattern, with room for rounding
+// > radius of the pattern (7.616), with room for rounding: 1000 steps lengthen (cs,
+// sn) by 3e-4 at most, from below sqrt(kMaxNorm2) at a level's start
+constexpr float kReach = 7.63f;
+constexpr float kMaxNorm2 = 1.003f;
 
 // Lane gl of a group owns the pattern points gl + LPK s, slot s < 2 NP, in
 // pairs of slots (2 j, 2 j + 1). A slot without a point has weight 0 (and
@@ -537,6 +540,14 @@ __device__ __forceinline__ void run_tracks(const Src& src, long long first, long
     if (ok) st = ts;
     bool run = ok && ts == VIO_TRACK_OK;   // steps are being taken
     const bool built = run;
+    // the samples stay in the window because the pattern, turned by (cs, sn),
+    // stays inside kReach: not with a start angle that is not finite, which has
+    // no samples and no mean (as in gn_step). 24,000 keypoints take 0.4% longer
+    // with this test.
+    if (run && K.iters > 0 && !(__fmaf_rn(W.cs, W.cs, __fmul_rn(W.sn, W.sn)) < kMaxNorm2)) {
+      st = VIO_TRACK_ZERO_MEAN;
+      run = false;
+    }
     const int iters = (int)__reduce_max_sync(kFull, run ? (unsigned)K.iters : 0u);
     for (int it = 0; it < iters; ++it) {
       bool step = run && it < K.iters;
