@@ -130,11 +130,12 @@ __global__ void __launch_bounds__(NT, 768 / NT) frame_front_kernel(const __grid_
       pyr::pyramid_pass(a.g, a.all, img, 0, a.m, a.T, tx, ty, a.ntx, a.nty, a.round_mode, smem);
     return;
   }
-  det::detect_block<MASKED>(level_ptr(a.g, a.all, base, 0), a.g.w[0], a.g.h[0], a.g.pitch[0],
-                            a.cg, a.gy, rem - n_pyr,
-                            MASKED ? a.mask + (long long)unit * a.mask_stride : nullptr,
-                            a.cand + (long long)unit * a.n_cells * a.cg.k,
-                            a.cand_count + (long long)unit * a.n_cells, smem);
+  if (a.n_cells > 0)
+    det::detect_block<MASKED>(level_ptr(a.g, a.all, base, 0), a.g.w[0], a.g.h[0], a.g.pitch[0],
+                              a.cg, a.gy, rem - n_pyr,
+                              MASKED ? a.mask + (long long)unit * a.mask_stride : nullptr,
+                              a.cand + (long long)unit * a.n_cells * a.cg.k,
+                              a.cand_count + (long long)unit * a.n_cells, smem);
   // after the level launches of a split front (a no-op otherwise): they read
   // the same frames and write nothing this launch reads, so it ran beside them
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -724,8 +725,10 @@ K1Args front_args(const vio_params& p, const Geom& g, const Batch& all, int det_
   a.cg = det::CellGeom{p.cell_w, p.cell_h, gx, p.k_per_cell, p.thresholds[p.n_thresholds - 1],
                        p.detect_border, 1, 1, 1, p.select_mode};
   det::detect_setup(a.cg, threads, det_warps);
-  a.blocks_per_unit = (a.m > 0 ? det_step * a.ntx * a.nty : 0) +
-                      (a.n_cells > 0 ? det::detect_blocks(gx, gy, a.cg.bcx, a.cg.bcy) : 0);
+  // at least one block: the group's first one counts its steps
+  a.blocks_per_unit = std::max(1, (a.m > 0 ? det_step * a.ntx * a.nty : 0) +
+                                      (a.n_cells > 0 ? det::detect_blocks(gx, gy, a.cg.bcx, a.cg.bcy)
+                                                     : 0));
   a.mask = mask;
   a.mask_stride = mask_stride;
   a.cand = cand;
