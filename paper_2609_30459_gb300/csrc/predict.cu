@@ -24,19 +24,38 @@ struct PredictArgs {
   uint8_t* valid;         // [img][cap], or null
 };
 
+// Every product that meets a sum is an explicit FMA or an unfused product, so
+// that the two kernels below round alike and a keypoint's start does not depend
+// on the size of its launch. Left to the compiler, the unrolled points of a
+// thread were contracted another way than a lane's: same positions, other last
+// bits of the angle (error against 64 bits over 6000 keypoints, mean 6.9e-7
+// rad, 6.3e-7 so).
+
 // Projection of the source pixel (x, y) at depth z into the target; false if
 // it is not in front of the target camera.
 __device__ __forceinline__ bool project(const PredictArgs& a, const vio_pose& T, float x, float y,
                                         float z, float& u, float& v) {
-  const float X = (x - a.ks.cx) * (z / a.ks.fx), Y = (y - a.ks.cy) * (z / a.ks.fy);
-  const float qx = T.R[0] * X + T.R[1] * Y + T.R[2] * z + T.t[0];
-  const float qy = T.R[3] * X + T.R[4] * Y + T.R[5] * z + T.t[1];
-  const float qz = T.R[6] * X + T.R[7] * Y + T.R[8] * z + T.t[2];
+  const float X = __fmul_rn(x - a.ks.cx, z / a.ks.fx), Y = __fmul_rn(y - a.ks.cy, z / a.ks.fy);
+  auto row = [&](int i) {
+    return __fadd_rn(__fadd_rn(__fmaf_rn(T.R[3 * i], X, __fmul_rn(T.R[3 * i + 1], Y)),
+                               __fmul_rn(T.R[3 * i + 2], z)),
+                     T.t[i]);
+  };
+  const float qx = row(0), qy = row(1), qz = row(2);
   if (!(qz > 0.f)) return false;
   const float iz = 1.f / qz;
-  u = a.kd.fx * qx * iz + a.kd.cx;
-  v = a.kd.fy * qy * iz + a.kd.cy;
+  u = __fmaf_rn(__fmul_rn(a.kd.fx, qx), iz, a.kd.cx);
+  v = __fmaf_rn(__fmul_rn(a.kd.fy, qy), iz, a.kd.cy);
   return true;
+}
+
+// A point's terms of the two sums: pattern offset (u, v), projected offset
+// (dx, dy).
+__device__ __forceinline__ float dot_term(float u, float v, float dx, float dy) {
+  return __fmaf_rn(u, dx, __fmul_rn(v, dy));
+}
+__device__ __forceinline__ float cross_term(float u, float v, float dx, float dy) {
+  return __fmaf_rn(u, dy, -__fmul_rn(v, dx));
 }
 
 __global__ void predict_kernel(const __grid_constant__ PredictArgs a) {
@@ -64,8 +83,8 @@ __global__ void predict_kernel(const __grid_constant__ PredictArgs a) {
       float yx = tx, yy = ty;
       ok = project(a, T, px + u, py + v, z, yx, yy) && ok;
       const float dx = yx - tx, dy = yy - ty;
-      dot += u * dx + v * dy;
-      cross += u * dy - v * dx;
+      dot = __fadd_rn(dot, dot_term(u, v, dx, dy));
+      cross = __fadd_rn(cross, cross_term(u, v, dx, dy));
     }
     if (ok) th = atan2f(cross, dot);
   }
@@ -83,10 +102,8 @@ __global__ void predict_kernel(const __grid_constant__ PredictArgs a) {
 // The same by eight lanes per keypoint, for launches of few keypoints: one
 // thread's 52 projections, each with a division, are a chain of 4 us however
 // few there are. A lane projects seven of the points; the two sums take the
-// lanes' terms in the order of the points, as one thread does (the angles
-// still differ by some last bits, the compiler contracting the projections of
-// an unrolled row differently). us a launch, keypoints: a thread each / eight
-// lanes each:
+// lanes' terms in the order of the points, as one thread does: the same results
+// bit for bit. us a launch, keypoints: a thread each / eight lanes each:
 //   900: 6.5 / 3.4    3000: 6.7 / 3.7    9000: 6.7 / 4.5    15000: 6.7 / 5.8
 //   30000: 7.1 / 9.0    150000: 14.0 / 35.8 (the sums' exchanges)
 constexpr int kLanes = 8;
@@ -123,16 +140,16 @@ __global__ void predict_lanes_kernel(const __grid_constant__ PredictArgs a) {
         float yx = tx, yy = ty;
         ok = project(a, T, px + u, py + v, z, yx, yy) && ok;
         const float dx = yx - tx, dy = yy - ty;
-        d[r] = u * dx + v * dy;
-        c[r] = u * dy - v * dx;
+        d[r] = dot_term(u, v, dx, dy);
+        c[r] = cross_term(u, v, dx, dy);
       }
     }
     ok = __all_sync(mask, ok);
     float dot = 0.f, cross = 0.f;
 #pragma unroll
     for (int j = 0; j < trk::kNP; ++j) {
-      dot += __shfl_sync(mask, d[j / kLanes], j % kLanes, kLanes);
-      cross += __shfl_sync(mask, c[j / kLanes], j % kLanes, kLanes);
+      dot = __fadd_rn(dot, __shfl_sync(mask, d[j / kLanes], j % kLanes, kLanes));
+      cross = __fadd_rn(cross, __shfl_sync(mask, c[j / kLanes], j % kLanes, kLanes));
     }
     if (ok) th = atan2f(cross, dot);
   }
