@@ -469,6 +469,10 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
   uint16_t* scored = reinterpret_cast<uint16_t*>(wsm + S.w_scored);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsm + S.w_keys);
   const int n16 = S.map_bytes >> 4;
+  // the map words this warp scans and whose pixels it scores: an even share (by
+  // 32 words in turn one warp of a 20 x 20 cell had 32 of the 33: 9 images of
+  // 192 such cells, k = 4: 38.2 us, 32.9 so; 512 images of 752 x 480: 673, 665)
+  const int word0 = n16 * gw / G, word1 = n16 * (gw + 1) / G;
 
   // zero maps; per quad: lanes where the bound is defined (FAST ring inside
   // the image, inside the cell's ring region)
@@ -600,10 +604,10 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
         const unsigned pb = (unsigned)tp * 0x01010101u, plo = pb & 0x7f7f7f7fu;
         int fill = 0;
 #pragma unroll 1
-        for (int base = gw * 32; base < n16; base += GT) {
+        for (int base = word0; base < word1; base += 32) {
           const int i = base + lane;
           uint4 w = make_uint4(0u, 0u, 0u, 0u);
-          if (i < n16) w = reinterpret_cast<const uint4*>(umap)[i];
+          if (i < word1) w = reinterpret_cast<const uint4*>(umap)[i];
           unsigned h[4] = {bytes_ge(w.x, tb, tlo), bytes_ge(w.y, tb, tlo), bytes_ge(w.z, tb, tlo),
                            bytes_ge(w.w, tb, tlo)};
           if (tp < 256) {   // scored in an earlier round
@@ -689,10 +693,10 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
         }
       } else {
         // the 16-pixel words this warp scanned in pass B
-        for (int base = gw * 32; base < n16; base += GT) {
+        for (int base = word0; base < word1; base += 32) {
           const int i = base + lane;
 #pragma unroll 1
-          for (int j = 0; j < 16; ++j) consider(i < n16 ? test(16 * i + j) : 0ull);
+          for (int j = 0; j < 16; ++j) consider(i < word1 ? test(16 * i + j) : 0ull);
         }
       }
       // candidates of the whole cell (all g warps, all rounds so far)
