@@ -150,7 +150,9 @@ cudaError_t launch_detect(const vio_params& p, const Geom& g, const Batch& b,
   const int n_cells = a.cg.gx * a.gy;
   a.n_cells = n_cells;
   const int smem = det::detect_setup(
-      a.cg, det::kThreads, det::warps_per_cell((long long)n_cells * b.n, sm_count()));
+      a.cg, det::kThreads,
+      det::warps_per_cell((long long)n_cells * b.n, sm_count(),
+                          det::detect_warps_per_sm(p.cell_w, p.cell_h)));
   if (smem < 0) return cudaErrorInvalidValue;
   bool small = false;   // the detection launch leaves most of the GPU idle
   if (n_cells > 0) {

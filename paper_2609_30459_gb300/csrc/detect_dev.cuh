@@ -203,18 +203,31 @@ __host__ __device__ inline int detect_blocks(int gx, int gy, int bcx, int bcy) {
   return ((gx + bcx - 1) / bcx) * ((gy + bcy - 1) / bcy);
 }
 
-// Warps per cell for a launch of n_cells cells on n_sms SMs: enough warps in
-// flight to fill the GPU, the 24 per SM that are resident at once (six CTAs of
-// four warps by their registers). Pyramid and detection of 12 images of 117
-// cells of 50 x 50 pixels, k = 4: 114 us with two warps per cell (16 per SM
-// wanted), 95 us with four; with 32 per SM wanted the same, but the 2000 cells
-// of two 1920 x 1080 pairs take two waves (four steps 520 -> 545 us).
-inline int warps_per_cell(long long n_cells, int n_sms) {
-  const long long want = 24LL * n_sms;
+// Warps per cell for a launch of n_cells cells on n_sms SMs: enough to have
+// per_sm warps of each SM at work.
+inline int warps_per_cell(long long n_cells, int n_sms, int per_sm) {
+  const long long want = (long long)per_sm * n_sms;
   int g = 1;
   while (g < 8 && n_cells * g < want) g <<= 1;
   return g;
 }
+// Warps wanted per SM by a detection launch of its own: the 24 that are resident
+// at once (six CTAs of four warps by their registers), in small cells 16. us a
+// call, 16 / 24 wanted, where the two differ:
+//   2618 cells of 28x28: 23.7 / 20.8, k = 4 40.2 / 27.8, with masks 69.3 / 48.4
+//   2484 of 50x50: 29.9 / 28.4, 40.2 / 36.3, 179.2 / 100.0
+//   1500 of 37x32: 16.7 / 18.9, 20.8 / 23.3, 57.0 / 40.2
+//   2436 of 22x22: 23.2 / 20.2, 34.8 / 29.1, 51.2 / 39.8
+//   2496 of 20x20: 20.3 / 20.9, 27.1 / 29.0, 41.4 / 35.1
+//   1728 of 20x20: 17.4 / 20.6, 23.8 / 27.3, 27.1 / 32.7
+//   3600 of 16x16: 21.5 / 26.1, 32.5 / 41.7, 35.4 / 44.1
+inline int detect_warps_per_sm(int cw, int ch) { return cw * ch < 448 ? 16 : 24; }
+// By the front of a frame step, which has its pyramid's warps too: a step of 5
+// streams of 752x480 (1500 cells) takes 123 us with 16 wanted and 126 with 24,
+// of 15 with 60x60 cells 124 and 135, of three 1920x1080 276 and 281, of three
+// 640x480 with 16x16 cells 247 and 256; only large cells with several keypoints
+// are the other way (five 1920x1080, 60x60 cells, k = 2: 336 and 310).
+constexpr int kFrontWarpsPerSm = 16;
 
 // 16-bit lanes of a pair at image x = xp (lane 0) and xp + 2 (lane 1): all
 // ones in a lane iff lo <= its x <= hi

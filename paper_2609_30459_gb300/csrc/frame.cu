@@ -804,7 +804,9 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     for (int i = 0; i < n_groups; ++i)
       cells += (long long)fl[i].n_streams * (fl[i].g.w[0] / fl[i].p.cell_w) *
                (fl[i].g.h[0] / fl[i].p.cell_h);
-    const int gw = tune.det_warps > 0 ? tune.det_warps : det::warps_per_cell(cells, sm_count());
+    const int gw = tune.det_warps > 0
+                       ? tune.det_warps
+                       : det::warps_per_cell(cells, sm_count(), det::kFrontWarpsPerSm);
     for (int i = 0; i < n_groups; ++i) {
       const FrameLaunch& f = fl[i];
       K1Args a = front_args(f.p, f.g, f.cur, 2, nullptr, 0, f.cand, f.cand_count,
