@@ -422,9 +422,16 @@ __device__ __forceinline__ void eval_entries(const uint16_t* list, int e0, int e
 // round usually finds the strongest: over 300 cells of a 752 x 480 frame, 1.03
 // rounds, 136 bounds tightened and 50 pixels scored a cell (1.31 rounds and
 // 124 scored with steps of 24 from 24 below the largest bound and no second
-// bound). Where few corners are left (masks, several per cell) the steep tail
-// saves rounds: 12 masked images of 641 x 479, four per 50 x 50 cell, 118 us
-// against 142 us with 10/16 throughout.
+// bound).
+// With a mask the third is 2/16 of the second and the fourth the lowest: a cell
+// whose corners are masked scores every pixel, its list overflows and each
+// round then tests the whole map. us a call, masks over a third of the image,
+// steps of 24 / 6/16 throughout / 2/16 and the lowest:
+//   6 images of 641 x 479, 50 x 50 cells, k = 4: 51 / 56 / 45
+//   20 of 752 x 480, 82 x 82, k = 4: 118 / 126 / 102
+//   one of 1920 x 1080, 60 x 60, k = 1: 70 / 75 / 58
+// For k = 1 and a warp per cell the third stays at 6/16: where little is masked
+// (60 images of 752 x 480, 37 x 32 cells) 91 us against 103.
 __device__ __forceinline__ int scaled(int t, int T, int n) { return (((t + T) * n) >> 4) - T; }
 
 // Detection in one cell by warp gw of its g warps. st: the block's staged
@@ -724,7 +731,7 @@ __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int 
       if (n_found >= k || t <= 1) break;
       tp = t;
       t = max(scaled(t, T, down), 1);
-      down = 6;
+      down = !MASKED ? 6 : down < 11 ? 0 : (k > 1 || G > 1) ? 2 : 6;
     }
   }
   // top k of the cell: each warp's best k, then the best k of those (or,
