@@ -692,11 +692,29 @@ bool split_front(const Geom* g, const int* n_streams, int n_groups, int pyr_firs
 }
 
 // Slots of a step's tracking launch per SM from which it runs by groups of lanes
-// (track_group.cuh) instead of a warp per keypoint. Many slots of a step are
-// empty and many tracks end early, which costs a warp of its own little and a
-// group its turn: plain and learned steps of mixed batches took, groups / warps,
-// 524 / 413 us at 63 slots per SM (four steps), 323 / 253 at 139, 333 / 259 at
-// 154, 418 / 328 at 179.
+// (track_group.cuh) instead of a warp per keypoint. Counted as used are, of a
+// list's slots, at most two per keypoint that a frame can add: a stream keeps
+// about one, and raising a capacity alone does not change the kernel (counted
+// in full, a step of two 752 x 480 streams of 300 cells took 116 us with room
+// for 8000 keypoints, by groups, and 86 with a warp each).
+//
+// Many slots of a step are empty and many tracks end early, which costs a warp
+// of its own little and a group its turn. us a step with 2 slots a cell, groups
+// / warps; all cells textured, half of them, 15%:
+//   slots per SM
+//    66 (two 1920 x 1080):  149 / 161, 139 / 119, 117 / 90
+//   118 (12 of 752 x 480):  182 / 192, 138 / 143, 117 / 97
+//   118, learned start:     222 / 228, 192 / 184, 171 / 135
+//   132 (four 1920 x 1080): 257 / 266, 160 / 183, 134 / 113
+//   197 (20 of 752 x 480):  300 / 283, 215 / 193, 136 / 115
+//   197 (the same, 753 x 481): 322 / 278, 234 / 201, 150 / 126
+//   197, learned start:     310 / 319, 243 / 237, 196 / 148
+//   276 (7 of 640 x 480, 16 x 16 cells): 303 / 387, 221 / 246, 135 / 121
+//   280 (16 of four odd sizes): 469 / 499, 342 / 334, 219 / 191
+//   289 (16 of four sizes): 414 / 498, 296 / 323, 185 / 171
+//   289, learned start:     501 / 566, 364 / 385, 251 / 212
+// Below 200 the groups lose with half of the lists filled about what they gain
+// with all of them.
 constexpr long long kGroupSlotsPerSm = 200;
 
 // Levels the fused pass of K1 computes (the rest follow in further passes);
@@ -897,6 +915,7 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
   MultiK2 m2{};
   m2.n = n_groups;
   acc = 0;
+  long long used = 0;   // slots, as kGroupSlotsPerSm counts them
   for (int i = 0; i < n_groups; ++i) {
     const FrameLaunch& f = fl[i];
     m2.f[i] = f;
@@ -905,12 +924,15 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
     acc += 2LL * f.n_streams * f.cap +
            (tune.stereo_after ? 0LL : (long long)f.n_streams * n_cells * f.p.k_per_cell);
     m2.block_end[i] = acc;
+    const long long fresh = (long long)n_cells * f.p.k_per_cell;
+    used += f.n_streams * (2 * std::min<long long>(f.cap, 2 * fresh) +
+                           (tune.stereo_after ? 0 : fresh));
   }
   const int k2t = tune.k2_threads;
   const bool k2_small = acc <= (long long)kDependentMaxWarpsPerSm * sm_count();
   if (acc > 0) {
     const long long blocks2 = (acc * 32 + k2t - 1) / k2t;
-    if (acc >= kGroupSlotsPerSm * sm_count())
+    if (used >= kGroupSlotsPerSm * sm_count())
       frame_track_groups_kernel<<<(unsigned)trk::group_ctas(acc), trk::kGroupThreads, 0, s>>>(m2);
     else if (acc <= trk::team_ctas())   // one wave (track_team.cuh)
       frame_track_team_kernel<<<(unsigned)acc, trk::kTeamThreads, 0, s>>>(m2);
