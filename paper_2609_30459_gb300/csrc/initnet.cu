@@ -63,41 +63,6 @@ struct ExtractArgs {
   int vec;       // x is 16-byte aligned
 };
 
-// Pixels cx .. cx + 7 of row cy of a level as bytes, 0x80 (input value 0)
-// outside the level: from the three aligned words that cover them when the
-// level's rows start on 4-byte boundaries (a word that starts inside the level
-// ends inside the row's pitch), else byte by byte.
-__device__ __forceinline__ void half_row(const uint8_t* __restrict__ p, int w, int h, int pitch,
-                                         int cx, int cy, unsigned (&b)[2]) {
-  b[0] = b[1] = 0x80808080u;
-  if (cy < 0 || cy >= h) return;
-  const uint8_t* row = p + (long long)cy * pitch;
-  if (((reinterpret_cast<uintptr_t>(p) | (uintptr_t)pitch) & 3) == 0) {
-    const int x4 = cx & ~3;
-    unsigned v[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int x = x4 + 4 * k;
-      v[k] = x >= 0 && x < w ? __ldg(reinterpret_cast<const unsigned*>(row + x)) : 0x80808080u;
-    }
-    const unsigned sh = 8u * (unsigned)(cx - x4);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const unsigned a = __funnelshift_r(v[k], v[k + 1], sh);
-      const int in = w - cx - 4 * k;   // pixels of this word before the level's end
-      const unsigned keep = in >= 4 ? 0xffffffffu : (in <= 0 ? 0u : (1u << (8 * in)) - 1u);
-      b[k] = (a & keep) | (0x80808080u & ~keep);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int x = cx + k;
-      const unsigned v = x >= 0 && x < w ? (unsigned)__ldg(row + x) : 0x80u;
-      b[k >> 2] = (b[k >> 2] & ~(0xffu << (8 * (k & 3)))) | (v << (8 * (k & 3)));
-    }
-  }
-}
-
 // Network inputs, one warp per keypoint. Bound by its output (2 KB a
 // keypoint); each lane makes half a row (eight pixels, one 16-byte store) of
 // every channel, so that a warp's store is 512 consecutive bytes and its

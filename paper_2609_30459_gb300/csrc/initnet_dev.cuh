@@ -41,7 +41,7 @@ constexpr int PACKED_BYTES = OFF_B + N_BIAS * 4;
 constexpr int M_W1 = 0, M_B1 = 1152, M_W2 = 1184, M_B2 = 10400, M_W3 = 10432, M_B3 = 19648,
               M_W4 = 19680, M_B4 = 27872, M_W5 = 27936, M_B5 = 28128, N_MASTER = 28131;
 
-// Per-warp shared memory (bytes): activations with a zero border.
+// Bordered activations; the offsets are of extract_warp's buffer (bytes).
 constexpr int XP = 18;                   // input 16 + 2
 constexpr int H1P = 10;                  // 8 + 2
 constexpr int H2P = 6;                   // 4 + 2
@@ -117,7 +117,7 @@ __device__ __forceinline__ void fc_layer(const uint16_t* in, const uint16_t* W, 
   }
 }
 
-// Zero the borders (and the zero word) of a warp's activation buffers.
+// Zeroes extract_warp's buffer.
 __device__ __forceinline__ void clear_warp_smem(uint8_t* ws, int lane) {
   uint32_t* p = reinterpret_cast<uint32_t*>(ws);
   for (int i = lane; i < WARP_SMEM / 4; i += 32) p[i] = 0u;
@@ -126,7 +126,8 @@ __device__ __forceinline__ void clear_warp_smem(uint8_t* ws, int lane) {
 
 // Input of keypoint (px, py): for level l in (la, lb), the 16 x 16 integer
 // grid from round(p / 2^l) - 8, source then target, (v - 128) / 64, zero
-// outside the level; written bordered into ws + S_X.
+// outside the level; written bordered into ws + S_X. The plain form, a value at
+// a time: no kernel runs it, the host check of the inputs does.
 __device__ __forceinline__ void extract_warp(const Geom& g, const Batch& src, int src_img,
                                              const Batch& dst, int dst_img, float px, float py,
                                              int la, int lb, uint8_t* ws, int lane) {
@@ -153,6 +154,41 @@ __device__ __forceinline__ void extract_warp(const Geom& g, const Batch& src, in
 
 namespace vio {
 namespace net {
+
+// Pixels cx .. cx + 7 of row cy of a level as bytes, 0x80 (input value 0)
+// outside the level: from the three aligned words that cover them when the
+// level's rows start on 4-byte boundaries (a word that starts inside the level
+// ends inside the row's pitch), else byte by byte.
+__device__ __forceinline__ void half_row(const uint8_t* __restrict__ p, int w, int h, int pitch,
+                                         int cx, int cy, unsigned (&b)[2]) {
+  b[0] = b[1] = 0x80808080u;
+  if (cy < 0 || cy >= h) return;
+  const uint8_t* row = p + (long long)cy * pitch;
+  if (((reinterpret_cast<uintptr_t>(p) | (uintptr_t)pitch) & 3) == 0) {
+    const int x4 = cx & ~3;
+    unsigned v[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int x = x4 + 4 * k;
+      v[k] = x >= 0 && x < w ? __ldg(reinterpret_cast<const unsigned*>(row + x)) : 0x80808080u;
+    }
+    const unsigned sh = 8u * (unsigned)(cx - x4);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const unsigned a = __funnelshift_r(v[k], v[k + 1], sh);
+      const int in = w - cx - 4 * k;   // pixels of this word before the level's end
+      const unsigned keep = in >= 4 ? 0xffffffffu : (in <= 0 ? 0u : (1u << (8 * in)) - 1u);
+      b[k] = (a & keep) | (0x80808080u & ~keep);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int x = cx + k;
+      const unsigned v = x >= 0 && x < w ? (unsigned)__ldg(row + x) : 0x80u;
+      b[k >> 2] = (b[k >> 2] & ~(0xffu << (8 * (k & 3)))) | (v << (8 * (k & 3)));
+    }
+  }
+}
 
 // Prefetch of one input row into registers, so that the loads of the next
 // group are in flight while the current one computes: the five aligned

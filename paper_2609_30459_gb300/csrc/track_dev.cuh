@@ -133,14 +133,6 @@ struct Lv {
   int w, h, pitch;
 };
 
-template <int N>
-__device__ __forceinline__ void warp_sum(float (&v)[N]) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-}
-
 // Sums four values over the warp and gives every lane all four totals, by a
 // transposed butterfly: after the xor-16 and xor-8 rounds each lane carries one
 // of the four partial sums (value 2*bit4 + bit3 of its lane id), three more xor
