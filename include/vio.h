@@ -17,7 +17,11 @@
  *  - Arguments are validated on the host before anything is enqueued. A call
  *    that returns non-zero has enqueued nothing, except VIO_ERR_CUDA, which
  *    reports a launch error from the CUDA runtime.
- *  - Images are uint8, row-major, with a row pitch in bytes. Pixel centres
+ *  - Images are uint8, row-major, with a row pitch in bytes. Rows are read in
+ *    aligned words of up to 16 bytes that hold at least one pixel of the row:
+ *    bytes behind a row's last pixel, up to the end of such a word and never
+ *    past the pitch, may be read, behind the last row too, and are not used.
+ *    Pixel centres
  *    are at integer coordinates; level-l coordinates are level-0 coordinates
  *    divided by 2^l. Keypoints are float32 (x, y) in level-0 pixels.
  *  - Batches: calls work on n_images images of one size at fixed strides
@@ -242,7 +246,10 @@ enum { VIO_TRACK_FORWARD = 0, VIO_TRACK_WITH_FB = 1 };
  * patches with an SE(2) warp (t_x, t_y, theta), coarse to fine, gn_iters
  * Gauss-Newton steps per level, from pyramid src[i] to dst[i]. The warp maps
  * pattern offset x to R(theta) x + t; t is the keypoint's position in the
- * target. One warp of 32 threads tracks one keypoint.
+ * target. Each keypoint is tracked by two warps (calls of up to 10 keypoints
+ * per SM), by four lanes (from 28 per SM; 48 where level 0 has rows that do
+ * not start on 4-byte boundaries) or by one warp (between); the results are
+ * the same bit for bit.
  *   d_pts:    per image `capacity` float2 source positions (image stride
  *             capacity), level-0 px.
  *   d_init:   per keypoint float3 starting warp (t_x, t_y, theta), same
@@ -528,10 +535,11 @@ typedef struct {
 
 /* Tunables of a batch step: threads per block of the tracking launches (32,
  * 64, 128, 256 or 512) where one warp tracks one keypoint (steps of 10 to 200
- * keypoint slots per SM, and the stereo matching after selection; smaller
- * steps give a keypoint two warps, larger ones four lanes, each at a block
- * size of its own), the pyramid tile scale (-1, 0, 1: half, default, double
- * the deepest-level tile side), the order of stereo matching (0: every
+ * keypoint slots per SM, room beyond two per keypoint that a frame can add
+ * not counted, and the stereo matching after selection; smaller steps give a
+ * keypoint two warps, larger ones four lanes, each at a block size of its
+ * own), the pyramid tile scale of the fused launch (-1, 0, 1: half, default,
+ * double the deepest-level tile side), the order of stereo matching (0: every
  * cell's candidates are matched beside temporal tracking; 1: only the
  * selected keypoints are matched, after selection, in two more launches),
  * the pyramid levels the fused pyramid+detection launch computes (1..4,

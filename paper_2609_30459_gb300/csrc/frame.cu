@@ -842,7 +842,7 @@ cudaError_t launch_frames(const FrameLaunch* fl, int n_groups, const FrameTune& 
       smem1 = sm > smem1 ? sm : smem1;
     }
     // beside one another as programmatic dependents, while the detection is
-    // about one wave of CTAs (two 1920 x 1080 pairs, pipelined over four frames:
+    // eight CTAs per SM at most (six are resident at once; two 1920 x 1080 pairs, pipelined over four frames:
     // 734 to 715 us; the batch's 2240 CTAs: 675 us so, 699 us beside)
     bool beside = split && acc <= 8LL * sm_count();
     for (int lv = 0; split; ++lv) {

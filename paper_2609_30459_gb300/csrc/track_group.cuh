@@ -1,5 +1,6 @@
 // The patch tracker by groups of lanes: a warp tracks 32 / LPK keypoints at a
-// time, LPK lanes (4, 8 or 16) each. Same arithmetic as the per-warp form of
+// time, LPK lanes (4, 8 or 16) each; the kernels use 4 (kGroupLanes), the host
+// check 16 too. Same arithmetic as the per-warp form of
 // track_dev.cuh, bit for bit: a lane that owns the pattern points i, i + LPK,
 // i + 2 LPK, ... adds locally what the per-warp form's first reduction rounds
 // add across lanes, in the same order, so only the last rounds remain as
