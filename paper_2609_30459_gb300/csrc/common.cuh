@@ -97,7 +97,9 @@ inline cudaError_t launch_dependent(K kernel, dim3 grid, unsigned block, size_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();   // reported once: not to the next call too
+  return e;
 }
 
 // The detection parameters of vio_params (cells, k, thresholds, border), as
