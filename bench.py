@@ -54,7 +54,7 @@ TRACK_NCU = {"profile": "profiles/tracking_launches.md"}
 # from an ncu capture of 512 images of the headline sequence with the L2 kept
 # between launches (profiles/pyramid_detect_752x480x512.md names the command);
 # a full launch moves this per image
-PYRDET_TRAFFIC_PER_IMAGE = 694718
+PYRDET_TRAFFIC_PER_IMAGE = 689779
 
 
 def seq_seed(rank: int) -> int:

@@ -456,10 +456,10 @@ __device__ __forceinline__ int scaled(int t, int T, int n) { return (((t + T) * 
 //
 // What bounds it: instructions, 2.7 thousand of a warp for a 37 x 32 cell (46%
 // staging, set-up and pass A, 16% the scan, 19% bounds and scores, the rest
-// tests, later rounds and the selection), issued at 62% of the rate; the loops
+// tests, later rounds and the selection), issued at 67% of the rate; the loops
 // are not unrolled because the warps of an SM, each in another phase, miss in
 // the instruction cache. 185 images of 752 x 480: 294 us with a scan of eight
-// pixels a word, prefix sums for the queue and every queued pixel scored; 195
+// pixels a word, prefix sums for the queue and every queued pixel scored; 187
 // us so.
 template <bool MASKED>
 __device__ __forceinline__ void detect_cell(const uint8_t* __restrict__ st, int rs, int sxa,

@@ -681,9 +681,18 @@ __global__ void __launch_bounds__(K3_THREADS)
 // beside the detection blocks. The fused launch saves launches where they
 // are the time (one 752 x 480 frame: 15 us against 28 us in four launches),
 // but recomputes halos and runs both parts at the larger one's shared memory
-// and registers: the 16 mixed streams of a batch (29 million pixels) took 301
-// us fused, 97 us split; two 1920 x 1080 pairs (8 million) 75 and 58 us. Only
-// when the levels of the fused pass are left to this rule (pyr_first 0).
+// and registers. us a whole step, split / fused with 256 threads / with 128:
+//   0.7 Mi pixels (one 752 x 480 stream): 61 / 57 / 57
+//   1.4 (two): 73 / 74 / 72    2.1 (three): 97 / 96 / 91
+//   2.8 (four): 112 / 111 / 109    3.4 (five): 120 / 123 / 119
+//   3.5 (two of 1280 x 720): 146 / 148 / 151
+//   4.0 (one of 1480 x 1420): 135 / 148 / 154
+//   4.1 (six of 752 x 480): 145 / 148 / 146
+//   4.1 (28 of 320 x 240): 136 / 143 / 135
+//   5.3 (three of 1280 x 720): 183 / 202 / 199
+//   7.9 (two of 1920 x 1080): 203 / 234 / 233
+//   27.9 (16 of four sizes): 492 / 698 / 631
+// Only when the levels of the fused pass are left to this rule (pyr_first 0).
 constexpr long long kSplitPixels = 4LL << 20;
 bool split_front(const Geom* g, const int* n_streams, int n_groups, int pyr_first) {
   long long px = 0;

@@ -16,7 +16,7 @@
 // region and a 24-row window of the target are copied asynchronously. The
 // window has 2 to 5 pixels of play; a step whose samples might leave it copies
 // it again around the current position. 58 instructions a keypoint and step.
-// What is left are dependent instructions at three warps per scheduler (163
+// What is left are dependent instructions at three warps per scheduler (162
 // registers a thread) and the instruction cache.
 //
 // Measured (640 x 480, five levels, five steps, forward and backward, us;
@@ -650,7 +650,7 @@ __device__ __forceinline__ void run_tracks(const Src& src, long long first, long
 }
 
 // Lanes per keypoint of the launches, and the warps of a launch over `total`
-// items: at most what the GPU holds at 163 registers a thread, then few enough
+// items: at most what the GPU holds at 162 registers a thread, then few enough
 // that every group gets about as many.
 constexpr int kGroupLanes = 4;
 constexpr int kGroupThreads = 64;   // CTA size
